@@ -5,9 +5,9 @@
 // backward, weight-gradient accumulation across tiles in tensor memory) process tiles
 // of 128 constraint rows.  Every GEMM is one or more tcgen05.mma of M = 128 issued by one
 // thread; operands are staged in shared memory in the canonical no-swizzle K-major
-// layout (tc.cuh); transposed operands of the weight gradients are written transposed
-// by the epilogue threads, so every MMA reads K-major tiles.  Adam runs on FP32 master
-// weights (mlp_adam_kernel) and refreshes the BF16 copies the GEMMs read.
+// layout (tc.cuh), and the products that need an operand transposed read the same tile
+// MN-major.  The blocks' partial gradients are added, and Adam runs on FP32 master
+// weights and refreshes the BF16 copies the GEMMs read, in mlp_reduce_kernel.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -65,15 +65,14 @@ struct MlpDev {
   const float* b3;
 };
 
-__device__ __forceinline__ float silu(float z) {
+__device__ __forceinline__ float sigmoid(float z) {
   float t;
   asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * z));
-  return z * fmaf(0.5f, t, 0.5f);
+  return fmaf(0.5f, t, 0.5f);
 }
+__device__ __forceinline__ float silu(float z) { return z * sigmoid(z); }
 __device__ __forceinline__ float silu_grad(float z) {
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * z));
-  const float s = fmaf(0.5f, t, 0.5f);
+  const float s = sigmoid(z);
   return s * (1.f + z * (1.f - s));
 }
 
@@ -108,16 +107,6 @@ __device__ void stage_kmajor(uint8_t* dst, const __nv_bfloat16* src, int rows, i
     st_shared_v4(base + tc::kmajor_off(m, kc, K), v.x, v.y, v.z, v.w);
   }
 }
-// Same, transposed: dst holds src^T ([K][rows] K-major over `rows`).
-__device__ void stage_kmajor_t(uint8_t* dst, const __nv_bfloat16* src, int rows, int K) {
-  const uint32_t base = tc::smem_u32(dst);
-  for (int e = threadIdx.x; e < rows * K; e += blockDim.x) {
-    const int m = e / K, k = e % K;
-    const __nv_bfloat16 v = src[(size_t)m * K + k];
-    st_shared_u16(base + tc::kmajor_off(k, m, rows), *reinterpret_cast<const uint16_t*>(&v));
-  }
-}
-
 struct InferSmem {
   uint8_t w1[kHid * kInPad * 2];
   uint8_t w2[kHid * kHid * 2];
@@ -280,58 +269,102 @@ __global__ void __launch_bounds__(128) mlp_wait_selftest_kernel(uint32_t polls, 
   if (warp == 0) tc::tmem_dealloc(tmem_addr, 32);
 }
 
+// ------------------------------------------------------------------ training
+// One tile of 128 rows needs five GEMMs: Z1 = X W1^T, Z2 = H1 W2^T, dH1 = dZ2 W2,
+// dW2 = dZ2^T H1, dW1 = dZ1^T X.  Every operand is staged once, as K-major core matrices
+// of the row-major matrix; the products that need it transposed read the same bytes as an
+// MN-major operand (tc::make_idesc_bf16 and tc::mn_desc), so nothing is stored twice.
+// What bounds a block: the chain load -> MMA -> SiLU -> MMA -> SiLU -> MMA -> SiLU' -> MMA
+// of its tile (a minibatch of 16384 rows is 128 tiles, one per SM).  Sixteen warps share
+// every epilogue, four threads per row with 32 columns each, so that a phase is 32 columns
+// long and the SM's tanh unit (3 x 128 evaluations per row) is what it waits for.  The
+// column sums (db1, db2, dw3, of the unrounded FP32 values) are taken by a transposing
+// butterfly in every warp.  Each block stores its partial gradients as they lie in its
+// registers (lanes = rows, 16 bytes each: coalesced), and mlp_reduce_kernel adds the
+// blocks' partials in a fixed order: no atomics, and a run is reproducible.
+// Measured, one Adam step on 16384 rows: 1481 us with a thread per row, transposed operand
+// copies written two bytes at a time, and the column sums and gradients by FP32 atomics
+// (shared memory: a compare-and-swap loop with all 128 threads on one address); 22.7
+// us now.
 namespace {
 
+constexpr int kTrainThreads = 512;
 struct TrainSmem {
-  uint8_t w1[kHid * kInPad * 2];   // W1 [h1][in]
-  uint8_t w2[kHid * kHid * 2];     // W2 [h2][h1]
-  uint8_t w2t[kHid * kHid * 2];    // W2^T [h1][h2]
-  uint8_t x[kTile * kInPad * 2];   // X [row][in]
-  uint8_t xt[kInPad * kTile * 2];  // X^T [in][row]
-  uint8_t h[kTile * kHid * 2];     // H1 [row][h1], later dZ2 [row][h2]
-  uint8_t ht[kHid * kTile * 2];    // H1^T [h1][row]
-  uint8_t dt[kHid * kTile * 2];    // dZ2^T [h2][row], later dZ1^T [h1][row]
+  uint8_t w1[kHid * kInPad * 2];  // W1 [h1][in]
+  uint8_t w2[kHid * kHid * 2];    // W2 [h2][h1]
+  uint8_t x[kTile * kInPad * 2];  // X [row][in]
+  uint8_t h[kTile * kHid * 2];    // H1 [row][h1]
+  uint8_t d[kTile * kHid * 2];    // dZ2 [row][h2], then dZ1 [row][h1]
   float b1[kHid], b2[kHid], w3[kHid];
-  float gb1[kHid], gb2[kHid], gw3[kHid];
-  float gb3, loss;
+  float part[4][kTile];           // shares of y per column quarter
+  float sums[3][4][kHid];         // db1, db2, dw3 per lane quarter
+  float gb3[4], loss[4];
   uint64_t mbar;
   uint64_t drain;  // drain_mma: arrives once every MMA issued so far has completed
   uint32_t tmem;
 };
 
+// Partial gradients of one block, in 16-byte units: dW2 as [column / 4][row], dW1 as
+// [column / 4][row] (24 columns), then db1, db2, dw3, and (db3, loss, 0, 0).
+constexpr int kPartW1 = kHid / 4 * kHid;
+constexpr int kPartB1 = kPartW1 + kIn / 4 * kHid;
+constexpr int kPartB2 = kPartB1 + kHid / 4;
+constexpr int kPartW3 = kPartB2 + kHid / 4;
+constexpr int kPartB3 = kPartW3 + kHid / 4;
+constexpr int kPart4 = kPartB3 + 1;
+
+// Sum over the warp's lanes of each of 32 values: lane l returns the sum of v[l].
+// Recursive halving: 31 shuffles instead of 32 x 5.
+__device__ __forceinline__ float column_sum(float (&v)[32], int lane) {
+#pragma unroll
+  for (int w = 16; w >= 1; w >>= 1) {
+    const bool up = (lane & w) != 0;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const float keep = up ? v[i + w] : v[i], send = up ? v[i] : v[i + w];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+    }
+  }
+  return v[0];
+}
+
 }  // namespace
 
-// Accumulates the gradient of L = sum_r (y_r - target_r)^2 * scale over `rows` rows into
-// grad[kNumParams] (FP32, atomically) and L into *loss.
-__global__ void __launch_bounds__(128, 1) mlp_train_kernel(const __nv_bfloat16* __restrict__ feat,
-                                                           const float* __restrict__ target,
-                                                           long long rows, float scale, MlpDev w,
-                                                           float* __restrict__ grad,
-                                                           float* __restrict__ loss, int* err) {
+// Gradient of L = sum_r (y_r - target_r)^2 * scale: block b's share over its tiles goes to
+// part[b * kPart4 ..].
+__global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_kernel(const __nv_bfloat16* __restrict__ feat,
+                                                                    const float* __restrict__ target,
+                                                                    long long rows, float scale, MlpDev w,
+                                                                    float4* __restrict__ part, int* err) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-  const int t = threadIdx.x, warp = t >> 5;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int quad = warp & 3, quarter = warp >> 2;
+  const int row = quad * 32 + lane;  // the TMEM lane (tile row) this thread reads
+  const int col = quarter * 32;      // first of its 32 columns
   if (warp == 0) tc::tmem_alloc(&S.tmem, 512);
-  if (t == 0) { tc::mbar_init(&S.mbar, 1); tc::mbar_init(&S.drain, 1); S.gb3 = 0.f; S.loss = 0.f; }
+  if (t == 0) { tc::mbar_init(&S.mbar, 1); tc::mbar_init(&S.drain, 1); }
+  const long long ntiles = (rows + kTile - 1) / kTile;
+  // a tile is 128 rows x 4 chunks of 16 bytes, one per thread; row t / 4, chunk t % 4
+  auto load_x = [&](long long tile) {
+    const long long r = tile * kTile + (t >> 2);
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (tile < ntiles && r < rows) v = reinterpret_cast<const uint4*>(feat + r * kInPad)[t & 3];
+    return v;
+  };
+  uint4 xv = load_x(blockIdx.x);
   stage_kmajor(S.w1, w.w1, kHid, kInPad);
   stage_kmajor(S.w2, w.w2, kHid, kHid);
-  stage_kmajor_t(S.w2t, w.w2, kHid, kHid);
-  S.b1[t] = w.b1[t]; S.b2[t] = w.b2[t]; S.w3[t] = w.w3[t];
-  S.gb1[t] = 0.f; S.gb2[t] = 0.f; S.gw3[t] = 0.f;
+  if (t < kHid) { S.b1[t] = w.b1[t]; S.b2[t] = w.b2[t]; S.w3[t] = w.w3[t]; }
   const float b3 = w.b3[0];
-  tc::fence_proxy_async();
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = S.tmem;
-  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
   const uint32_t T_Z1 = 0, T_Z2 = 128, T_DW1 = 256, T_DW2 = 384;  // TMEM columns
-  const uint32_t id_128 = tc::make_idesc_bf16(kTile, kHid);
-  const uint32_t id_32 = tc::make_idesc_bf16(kHid, kInPad);
-  const uint32_t sx = tc::smem_u32(S.x), sxt = tc::smem_u32(S.xt), sh = tc::smem_u32(S.h);
-  const uint32_t sht = tc::smem_u32(S.ht), sdt = tc::smem_u32(S.dt);
-  const uint32_t sw1 = tc::smem_u32(S.w1), sw2 = tc::smem_u32(S.w2), sw2t = tc::smem_u32(S.w2t);
+  const uint32_t id_kk = tc::make_idesc_bf16(kTile, kHid);
+  const uint32_t id_kn = tc::make_idesc_bf16(kTile, kHid, false, true);
+  const uint32_t id_nn = tc::make_idesc_bf16(kHid, kHid, true, true);
+  const uint32_t id_nn32 = tc::make_idesc_bf16(kHid, kInPad, true, true);
+  const uint32_t sx = tc::smem_u32(S.x), sh = tc::smem_u32(S.h), sd = tc::smem_u32(S.d);
+  const uint32_t sw1 = tc::smem_u32(S.w1), sw2 = tc::smem_u32(S.w2);
   const uint32_t SB32 = kInPad / 8 * 128, SB128 = kHid / 8 * 128;
   uint32_t phase = 0;
   bool ok = true, first = true;
@@ -350,171 +383,215 @@ __global__ void __launch_bounds__(128, 1) mlp_train_kernel(const __nv_bfloat16* 
     tc::fence_after_sync();
     return true;
   };
-  const long long ntiles = (rows + kTile - 1) / kTile;
+  float gb1 = 0.f, gb2 = 0.f, gw3 = 0.f;  // column col + lane, rows of this warp's quarter
+  float gb3 = 0.f, loss = 0.f;            // this thread's row (column quarter 0 only)
+  st_shared_v4(sx + tc::kmajor_off(t >> 2, 8 * (t & 3), kInPad), xv.x, xv.y, xv.z, xv.w);
+  sync_mma();
+  const uint32_t tmem = S.tmem;
+  const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const long long r = tile * kTile + t;
-    const bool valid = r < rows;
-    // X row -> sX (K-major over inputs) and X^T -> sXT (K-major over rows)
-    uint4 v[4] = {};
-    if (valid) {
-      const uint4* src = reinterpret_cast<const uint4*>(feat + r * kInPad);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] = src[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      st_shared_v4(sx + tc::kmajor_off(t, 8 * q, kInPad), v[q].x, v[q].y, v[q].z, v[q].w);
-      const uint16_t* e = reinterpret_cast<const uint16_t*>(&v[q]);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) st_shared_u16(sxt + tc::kmajor_off(8 * q + i, t, kTile), e[i]);
-    }
-    sync_mma();
     if (t == 0) {
+#pragma unroll
       for (int kk = 0; kk < kInPad / 16; ++kk)
         tc::mma_bf16(tmem + T_Z1, tc::make_sdesc(sx + kk * 256, 128, SB32),
-                     tc::make_sdesc(sw1 + kk * 256, 128, SB32), id_128, kk > 0);
+                     tc::make_sdesc(sw1 + kk * 256, 128, SB32), id_kk, kk > 0);
       tc::mma_commit(&S.mbar);
     }
+    const long long r = tile * kTile + row;
+    const bool valid = r < rows;
+    const float tg = valid ? target[r] : 0.f;
+    xv = load_x(tile + gridDim.x);
     if (!(ok = wait_mma())) break;
-    // H1 = silu(Z1 + b1) -> sH [row][h1] and sHT [h1][row]
-    for (int c0 = 0; c0 < kHid; c0 += 32) {
+    // H1 = silu(Z1 + b1)
+    {
       float a[32];
-      tc::tmem_ld32(tmem + lane_base + T_Z1 + c0, a);
+      tc::tmem_ld32(tmem + lane_base + T_Z1 + col, a);
+#pragma unroll
       for (int q = 0; q < 4; ++q) {
         uint32_t p[4];
+#pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const int c = c0 + 8 * q + 2 * e;
-          p[e] = pack_bf16x2(silu(a[8 * q + 2 * e] + S.b1[c]), silu(a[8 * q + 2 * e + 1] + S.b1[c + 1]));
+          const int i = 8 * q + 2 * e;
+          p[e] = pack_bf16x2(silu(a[i] + S.b1[col + i]), silu(a[i + 1] + S.b1[col + i + 1]));
         }
-        st_shared_v4(sh + tc::kmajor_off(t, c0 + 8 * q, kHid), p[0], p[1], p[2], p[3]);
-        const uint16_t* e16 = reinterpret_cast<const uint16_t*>(p);
-        for (int i = 0; i < 8; ++i) st_shared_u16(sht + tc::kmajor_off(c0 + 8 * q + i, t, kTile), e16[i]);
+        st_shared_v4(sh + tc::kmajor_off(row, col + 8 * q, kHid), p[0], p[1], p[2], p[3]);
       }
     }
     sync_mma();
     if (t == 0) {
+#pragma unroll
       for (int kk = 0; kk < kHid / 16; ++kk)
         tc::mma_bf16(tmem + T_Z2, tc::make_sdesc(sh + kk * 256, 128, SB128),
-                     tc::make_sdesc(sw2 + kk * 256, 128, SB128), id_128, kk > 0);
+                     tc::make_sdesc(sw2 + kk * 256, 128, SB128), id_kk, kk > 0);
       tc::mma_commit(&S.mbar);
     }
     if (!(ok = wait_mma())) break;
-    // y, loss, g = dL/dy
-    float y = b3;
-    for (int c0 = 0; c0 < kHid; c0 += 32) {
-      float a[32];
-      tc::tmem_ld32(tmem + lane_base + T_Z2 + c0, a);
-      for (int i = 0; i < 32; ++i) y = fmaf(S.w3[c0 + i], silu(a[i] + S.b2[c0 + i]), y);
-    }
-    const float res = valid ? y - target[r] : 0.f;
-    const float g = 2.f * res * scale;
-    atomicAdd(&S.loss, res * res * scale);
-    atomicAdd(&S.gb3, g);
-    // dZ2 = g w3 * silu'(Z2) -> sH [row][h2] and sDT [h2][row]; dw3 += g H2; db2 += dZ2
-    for (int c0 = 0; c0 < kHid; c0 += 32) {
-      float a[32];
-      tc::tmem_ld32(tmem + lane_base + T_Z2 + c0, a);
-      for (int q = 0; q < 4; ++q) {
-        uint32_t p[4];
-        for (int e = 0; e < 4; ++e) {
-          float d2[2];
-          for (int u = 0; u < 2; ++u) {
-            const int i = 8 * q + 2 * e + u, c = c0 + i;
-            const float z = a[i] + S.b2[c];
-            d2[u] = g * S.w3[c] * silu_grad(z);
-            if (valid) {
-              atomicAdd(&S.gw3[c], g * silu(z));
-              atomicAdd(&S.gb2[c], d2[u]);
-            }
-          }
-          p[e] = pack_bf16x2(d2[0], d2[1]);
-        }
-        st_shared_v4(sh + tc::kmajor_off(t, c0 + 8 * q, kHid), p[0], p[1], p[2], p[3]);
-        const uint16_t* e16 = reinterpret_cast<const uint16_t*>(p);
-        for (int i = 0; i < 8; ++i) st_shared_u16(sdt + tc::kmajor_off(c0 + 8 * q + i, t, kTile), e16[i]);
-      }
-    }
-    sync_mma();
-    if (t == 0) {
-      // dH1 = dZ2 W2  (into the Z2 columns, consumed)
-      for (int kk = 0; kk < kHid / 16; ++kk)
-        tc::mma_bf16(tmem + T_Z2, tc::make_sdesc(sh + kk * 256, 128, SB128),
-                     tc::make_sdesc(sw2t + kk * 256, 128, SB128), id_128, kk > 0);
-      // dW2 += dZ2^T H1
-      for (int kk = 0; kk < kTile / 16; ++kk)
-        tc::mma_bf16(tmem + T_DW2, tc::make_sdesc(sdt + kk * 256, 128, SB128),
-                     tc::make_sdesc(sht + kk * 256, 128, SB128), id_128, (!first || kk > 0) ? 1u : 0u);
-      tc::mma_commit(&S.mbar);
-    }
-    if (!(ok = wait_mma())) break;
-    // dZ1 = dH1 * silu'(Z1) -> sDT [h1][row]; db1 += dZ1
-    for (int c0 = 0; c0 < kHid; c0 += 32) {
-      float a[32], z1[32];
-      tc::tmem_ld32(tmem + lane_base + T_Z2 + c0, a);
-      tc::tmem_ld32(tmem + lane_base + T_Z1 + c0, z1);
+    // y, g = dL/dy, dZ2 = g w3 silu'(Z2) and the column sums dw3, db2
+    {
+      float z[32], s[32];
+      tc::tmem_ld32(tmem + lane_base + T_Z2 + col, z);
+      float y = 0.f;
+#pragma unroll
       for (int i = 0; i < 32; ++i) {
-        const int c = c0 + i;
-        const float d1 = a[i] * silu_grad(z1[i] + S.b1[c]);
-        const __nv_bfloat16 b = __float2bfloat16_rn(d1);
-        st_shared_u16(sdt + tc::kmajor_off(c, t, kTile), *reinterpret_cast<const uint16_t*>(&b));
-        if (valid) atomicAdd(&S.gb1[c], d1);
+        z[i] += S.b2[col + i];
+        s[i] = sigmoid(z[i]);
+        y = fmaf(S.w3[col + i], z[i] * s[i], y);
       }
+      S.part[quarter][row] = y;
+      __syncthreads();
+      y = b3 + ((S.part[0][row] + S.part[1][row]) + (S.part[2][row] + S.part[3][row]));
+      const float res = valid ? y - tg : 0.f;
+      const float g = 2.f * res * scale;
+      if (quarter == 0) { loss += res * res * scale; gb3 += g; }
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float h2 = z[i] * s[i];
+        s[i] = g * S.w3[col + i] * (s[i] * (1.f + z[i] * (1.f - s[i])));
+        z[i] = g * h2;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        st_shared_v4(sd + tc::kmajor_off(row, col + 8 * q, kHid), pack_bf16x2(s[8 * q], s[8 * q + 1]),
+                     pack_bf16x2(s[8 * q + 2], s[8 * q + 3]), pack_bf16x2(s[8 * q + 4], s[8 * q + 5]),
+                     pack_bf16x2(s[8 * q + 6], s[8 * q + 7]));
+      sync_mma();
+      if (t == 0) {
+        // dH1 = dZ2 W2 (into the Z2 columns, consumed); dW2 += dZ2^T H1
+#pragma unroll
+        for (int kk = 0; kk < kHid / 16; ++kk)
+          tc::mma_bf16(tmem + T_Z2, tc::make_sdesc(sd + kk * 256, 128, SB128),
+                       tc::mn_desc(sw2 + kk * 2 * SB128, SB128), id_kn, kk > 0);
+#pragma unroll
+        for (int kk = 0; kk < kTile / 16; ++kk)
+          tc::mma_bf16(tmem + T_DW2, tc::mn_desc(sd + kk * 2 * SB128, SB128),
+                       tc::mn_desc(sh + kk * 2 * SB128, SB128), id_nn, (!first || kk > 0) ? 1u : 0u);
+        tc::mma_commit(&S.mbar);
+      }
+      gw3 += column_sum(z, lane);  // while the tensor core works
+      gb2 += column_sum(s, lane);
     }
-    sync_mma();
-    if (t == 0) {
-      // dW1 += dZ1^T X
-      for (int kk = 0; kk < kTile / 16; ++kk)
-        tc::mma_bf16(tmem + T_DW1, tc::make_sdesc(sdt + kk * 256, 128, SB128),
-                     tc::make_sdesc(sxt + kk * 256, 128, SB128), id_32, (!first || kk > 0) ? 1u : 0u);
-      tc::mma_commit(&S.mbar);
+    if (!(ok = wait_mma())) break;
+    // dZ1 = dH1 silu'(Z1) and its column sums db1
+    {
+      float a[32], z[32];
+      tc::tmem_ld32(tmem + lane_base + T_Z2 + col, a);
+      tc::tmem_ld32(tmem + lane_base + T_Z1 + col, z);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) a[i] *= silu_grad(z[i] + S.b1[col + i]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        st_shared_v4(sd + tc::kmajor_off(row, col + 8 * q, kHid), pack_bf16x2(a[8 * q], a[8 * q + 1]),
+                     pack_bf16x2(a[8 * q + 2], a[8 * q + 3]), pack_bf16x2(a[8 * q + 4], a[8 * q + 5]),
+                     pack_bf16x2(a[8 * q + 6], a[8 * q + 7]));
+      sync_mma();
+      if (t == 0) {
+        // dW1 += dZ1^T X
+#pragma unroll
+        for (int kk = 0; kk < kTile / 16; ++kk)
+          tc::mma_bf16(tmem + T_DW1, tc::mn_desc(sd + kk * 2 * SB128, SB128),
+                       tc::mn_desc(sx + kk * 2 * SB32, SB32), id_nn32, (!first || kk > 0) ? 1u : 0u);
+        tc::mma_commit(&S.mbar);
+      }
+      gb1 += column_sum(a, lane);
     }
     if (!(ok = wait_mma())) break;
     first = false;
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
+    st_shared_v4(sx + tc::kmajor_off(t >> 2, 8 * (t & 3), kInPad), xv.x, xv.y, xv.z, xv.w);
+    sync_mma();
   }
   if (!ok) drain_mma(&S.drain, t);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  if (ok && !first) {
-    // weight gradients out of tensor memory: thread t owns row t of dW2 and dW1
-    for (int c0 = 0; c0 < kHid; c0 += 32) {
-      float a[32];
-      tc::tmem_ld32(tmem + lane_base + T_DW2 + c0, a);
-      for (int i = 0; i < 32; ++i) atomicAdd(&grad[kOffW2 + t * kHid + c0 + i], a[i]);
-    }
+  // this block's partial gradients (zeros after a timed-out wait, which is reported)
+  part += (size_t)blockIdx.x * kPart4;
+  const float on = ok ? 1.f : 0.f;
+  {
     float a[32];
-    tc::tmem_ld32(tmem + lane_base + T_DW1, a);
-    for (int i = 0; i < kIn; ++i) atomicAdd(&grad[kOffW1 + t * kIn + i], a[i]);
-    atomicAdd(&grad[kOffB1 + t], S.gb1[t]);
-    atomicAdd(&grad[kOffB2 + t], S.gb2[t]);
-    atomicAdd(&grad[kOffW3 + t], S.gw3[t]);
-    if (t == 0) { atomicAdd(&grad[kOffB3], S.gb3); atomicAdd(loss, S.loss); }
+    tc::tmem_ld32(tmem + lane_base + T_DW2 + col, a);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      part[(col / 4 + q) * kHid + row] =
+          ok ? make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (quarter == 0) {
+      tc::tmem_ld32(tmem + lane_base + T_DW1, a);
+#pragma unroll
+      for (int q = 0; q < kIn / 4; ++q)
+        part[kPartW1 + q * kHid + row] =
+            ok ? make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
+        loss += __shfl_xor_sync(0xffffffffu, loss, o);
+      }
+      if (lane == 0) { S.gb3[quad] = gb3; S.loss[quad] = loss; }
+    }
   }
+  S.sums[0][quad][col + lane] = gb1;
+  S.sums[1][quad][col + lane] = gb2;
+  S.sums[2][quad][col + lane] = gw3;
   tc::fence_before_sync();
   __syncthreads();
+  if (t < 3 * kHid) {
+    const int k = t / kHid, c = t % kHid;
+    reinterpret_cast<float*>(part + kPartB1)[t] =
+        on * ((S.sums[k][0][c] + S.sums[k][1][c]) + (S.sums[k][2][c] + S.sums[k][3][c]));
+  } else if (t == 3 * kHid) {
+    part[kPartB3] = make_float4(on * ((S.gb3[0] + S.gb3[1]) + (S.gb3[2] + S.gb3[3])),
+                                on * ((S.loss[0] + S.loss[1]) + (S.loss[2] + S.loss[3])), 0.f, 0.f);
+  }
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-// Adam on the FP32 master parameters; refreshes the BF16 weight copies.
-__global__ void mlp_adam_kernel(float* __restrict__ p, float* __restrict__ g, float* __restrict__ m,
-                                float* __restrict__ v, float lr, float b1, float b2, float eps,
-                                float c1, float c2, __nv_bfloat16* __restrict__ w1b,
-                                __nv_bfloat16* __restrict__ w2b) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kNumParams) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+// Adds the training blocks' partial gradients and writes the gradient (out, may be null) and
+// the loss (may be null); with p, one Adam step on the FP32 master parameters with it, which
+// refreshes the BF16 weight copies.  A block takes 32 of the kPart4 16-byte units: eight
+// warps add every eighth block's share (independent loads), the first four combine them.
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float4* __restrict__ part, int n_part,
+                                                         float* __restrict__ out, float* __restrict__ loss,
+                                                         float* __restrict__ p, float* __restrict__ m,
+                                                         float* __restrict__ v, float lr, float b1, float b2,
+                                                         float eps, float c1, float c2,
+                                                         __nv_bfloat16* __restrict__ w1b,
+                                                         __nv_bfloat16* __restrict__ w2b) {
+  __shared__ float4 sums[8][32];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  {
+    const int u = blockIdx.x * 32 + lane;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (u < kPart4)
+#pragma unroll 4
+      for (int b = warp; b < n_part; b += 8) {
+        const float4 q = part[(size_t)b * kPart4 + u];
+        a.x += q.x; a.y += q.y; a.z += q.z; a.w += q.w;
+      }
+    sums[warp][lane] = a;
+  }
+  __syncthreads();
+  if (t >= 128) return;
+  const int u = blockIdx.x * 32 + (t >> 2), k = t & 3;
+  if (u >= kPart4) return;
+  float g = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) g += reinterpret_cast<const float*>(&sums[w][t >> 2])[k];
+  int i;  // index in the parameter vector
+  if (u < kPartW1) i = kOffW2 + (u % kHid) * kHid + 4 * (u / kHid) + k;
+  else if (u < kPartB1) i = kOffW1 + ((u - kPartW1) % kHid) * kIn + 4 * ((u - kPartW1) / kHid) + k;
+  else if (u < kPartB2) i = kOffB1 + 4 * (u - kPartB1) + k;
+  else if (u < kPartW3) i = kOffB2 + 4 * (u - kPartB2) + k;
+  else if (u < kPartB3) i = kOffW3 + 4 * (u - kPartW3) + k;
+  else {
+    if (k == 1 && loss) *loss = g;
+    if (k != 0) return;
+    i = kOffB3;
+  }
+  if (out) out[i] = g;
+  if (!p) return;
+  const float mi = b1 * m[i] + (1.f - b1) * g;
+  const float vi = b2 * v[i] + (1.f - b2) * g * g;
   m[i] = mi; v[i] = vi;
   const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
   p[i] = pi;
-  g[i] = 0.f;
   if (i < kOffB1) {
-    const int o = i / kIn, k = i % kIn;
-    w1b[o * kInPad + k] = __float2bfloat16_rn(pi);
+    const int o = i / kIn, c = i % kIn;
+    w1b[o * kInPad + c] = __float2bfloat16_rn(pi);
   } else if (i >= kOffW2 && i < kOffB2) {
     w2b[i - kOffW2] = __float2bfloat16_rn(pi);
   }
@@ -538,9 +615,10 @@ SimStatus mlp_forward_launch(MlpHandle* h, const void* feat, long long rows, flo
 }
 struct MlpHandle {
   cudaStream_t stream = nullptr;
-  float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
+  uint8_t* mem = nullptr;  // owns the device buffers below
+  float *p = nullptr, *m = nullptr, *v = nullptr;
+  float4* part = nullptr;  // [sms][kPart4] partial gradients of the training blocks
   __nv_bfloat16 *w1b = nullptr, *w2b = nullptr;
-  float* loss = nullptr;
   int* err = nullptr;
   long long adam_t = 0;
   int sms = 0;
@@ -570,6 +648,17 @@ SimStatus check_err(MlpHandle* h) {
   if (e) return mfail(SIM_ECUDA, "tensor-core wait timed out");
   return SIM_OK;
 }
+
+// Partial gradients of `rows` rows (0: no blocks) into h->part; *grid receives the blocks.
+SimStatus train_launch(MlpHandle* h, const void* feat, const float* target, long long rows, float scale, int* grid) {
+  const long long tiles = (rows + kTile - 1) / kTile;
+  *grid = (int)std::min<long long>(tiles, h->sms);
+  if (*grid == 0) return SIM_OK;
+  mlp_train_kernel<<<*grid, kTrainThreads, sizeof(TrainSmem), h->stream>>>((const __nv_bfloat16*)feat, target, rows,
+                                                                          scale, dev_of(h), h->part, h->err);
+  MCU(cudaGetLastError());
+  return SIM_OK;
+}
 }  // namespace
 
 SimStatus snakesim::mlp_forward_launch(MlpHandle* h, const void* feat, long long rows, float* out,
@@ -590,27 +679,27 @@ SimStatus mlp_create(void* stream, MlpHandle** out) {
   *out = nullptr;
   MlpHandle* h = new MlpHandle();
   h->stream = (cudaStream_t)stream;
-  cudaError_t e = cudaSuccess;
-  auto alloc = [&](void** p, size_t b) { if (e == cudaSuccess) e = cudaMalloc(p, b); };
-  alloc((void**)&h->p, kNumParams * sizeof(float));
-  alloc((void**)&h->g, kNumParams * sizeof(float));
-  alloc((void**)&h->m, kNumParams * sizeof(float));
-  alloc((void**)&h->v, kNumParams * sizeof(float));
-  alloc((void**)&h->w1b, kHid * kInPad * sizeof(__nv_bfloat16));
-  alloc((void**)&h->w2b, kHid * kHid * sizeof(__nv_bfloat16));
-  alloc((void**)&h->loss, sizeof(float));
-  alloc((void**)&h->err, sizeof(int));
-  if (e != cudaSuccess) { mlp_destroy(h); return mfail(SIM_ENOMEM, cudaGetErrorString(e)); }
-  cudaMemset(h->p, 0, kNumParams * sizeof(float));
-  cudaMemset(h->g, 0, kNumParams * sizeof(float));
-  cudaMemset(h->m, 0, kNumParams * sizeof(float));
-  cudaMemset(h->v, 0, kNumParams * sizeof(float));
-  cudaMemset(h->w1b, 0, kHid * kInPad * sizeof(__nv_bfloat16));
-  cudaMemset(h->w2b, 0, kHid * kHid * sizeof(__nv_bfloat16));
-  cudaMemset(h->err, 0, sizeof(int));
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
+  // one allocation: the parameters, moments, weight copies and the flag (zeroed), then the
+  // training blocks' partial gradients (written before they are read)
+  size_t at = 0;
+  auto take = [&](size_t bytes) { const size_t o = at; at += (bytes + 255) & ~(size_t)255; return o; };
+  const size_t o_p = take(kNumParams * sizeof(float)), o_m = take(kNumParams * sizeof(float));
+  const size_t o_v = take(kNumParams * sizeof(float)), o_w1 = take(kHid * kInPad * sizeof(__nv_bfloat16));
+  const size_t o_w2 = take(kHid * kHid * sizeof(__nv_bfloat16)), o_err = take(sizeof(int));
+  const size_t zeroed = at, o_part = take((size_t)std::max(1, h->sms) * kPart4 * sizeof(float4));
+  cudaError_t e = cudaMalloc((void**)&h->mem, at);
+  if (e != cudaSuccess) { h->mem = nullptr; mlp_destroy(h); return mfail(SIM_ENOMEM, cudaGetErrorString(e)); }
+  h->p = (float*)(h->mem + o_p);
+  h->m = (float*)(h->mem + o_m);
+  h->v = (float*)(h->mem + o_v);
+  h->w1b = (__nv_bfloat16*)(h->mem + o_w1);
+  h->w2b = (__nv_bfloat16*)(h->mem + o_w2);
+  h->err = (int*)(h->mem + o_err);
+  h->part = (float4*)(h->mem + o_part);
+  cudaMemset(h->mem, 0, zeroed);
   e = cudaFuncSetAttribute(mlp_infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(InferSmem));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem));
@@ -652,17 +741,12 @@ SimStatus mlp_grad(MlpHandle* h, const void* feat, const float* target, int64_t 
                    float* grad, float* loss) {
   if (!h || !feat || !target || rows < 0) return mfail(SIM_EINVAL, "bad arguments");
   if (((uintptr_t)feat & 15u) != 0) return mfail(SIM_EINVAL, "feat is not 16-byte aligned");
-  MCU(cudaMemsetAsync(h->g, 0, kNumParams * sizeof(float), h->stream));
-  MCU(cudaMemsetAsync(h->loss, 0, sizeof(float), h->stream));
-  if (rows > 0) {
-    const long long tiles = (rows + kTile - 1) / kTile;
-    const int grid = (int)std::min<long long>(tiles, h->sms);
-    mlp_train_kernel<<<grid, 128, sizeof(TrainSmem), h->stream>>>((const __nv_bfloat16*)feat, target, rows,
-                                                                   scale, dev_of(h), h->g, h->loss, h->err);
-    MCU(cudaGetLastError());
-  }
-  if (grad) MCU(cudaMemcpyAsync(grad, h->g, kNumParams * sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
-  if (loss) MCU(cudaMemcpyAsync(loss, h->loss, sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
+  int grid = 0;
+  SimStatus s = train_launch(h, feat, target, rows, scale, &grid);
+  if (s != SIM_OK) return s;
+  mlp_reduce_kernel<<<(kPart4 + 31) / 32, 256, 0, h->stream>>>(h->part, grid, grad, loss, nullptr, nullptr, nullptr,
+                                                               0.f, 0.f, 0.f, 0.f, 1.f, 1.f, nullptr, nullptr);
+  MCU(cudaGetLastError());
   return check_err(h);
 }
 
@@ -670,20 +754,15 @@ SimStatus mlp_train_step(MlpHandle* h, const void* feat, const float* target, in
                          float* loss) {
   if (!h || !feat || !target || rows <= 0 || !(lr > 0.f)) return mfail(SIM_EINVAL, "bad arguments");
   if (((uintptr_t)feat & 15u) != 0) return mfail(SIM_EINVAL, "feat is not 16-byte aligned");
-  MCU(cudaMemsetAsync(h->g, 0, kNumParams * sizeof(float), h->stream));
-  MCU(cudaMemsetAsync(h->loss, 0, sizeof(float), h->stream));
-  const long long tiles = (rows + kTile - 1) / kTile;
-  const int grid = (int)std::min<long long>(tiles, h->sms);
-  mlp_train_kernel<<<grid, 128, sizeof(TrainSmem), h->stream>>>((const __nv_bfloat16*)feat, target, rows,
-                                                                 1.0f / (float)rows, dev_of(h), h->g, h->loss, h->err);
-  MCU(cudaGetLastError());
+  int grid = 0;
+  SimStatus s = train_launch(h, feat, target, rows, 1.0f / (float)rows, &grid);
+  if (s != SIM_OK) return s;
   h->adam_t += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)h->adam_t), c2 = 1.f - powf(b2, (float)h->adam_t);
-  mlp_adam_kernel<<<(kNumParams + 255) / 256, 256, 0, h->stream>>>(h->p, h->g, h->m, h->v, lr, b1, b2, 1e-8f,
-                                                                   c1, c2, h->w1b, h->w2b);
+  mlp_reduce_kernel<<<(kPart4 + 31) / 32, 256, 0, h->stream>>>(h->part, grid, nullptr, loss, h->p, h->m, h->v, lr, b1,
+                                                               b2, 1e-8f, c1, c2, h->w1b, h->w2b);
   MCU(cudaGetLastError());
-  if (loss) MCU(cudaMemcpyAsync(loss, h->loss, sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
   return SIM_OK;
 }
 
@@ -714,8 +793,7 @@ SimStatus mlp_wait_selftest(uint32_t polls, void* stream, int32_t* timed_out) {
 SimStatus mlp_destroy(MlpHandle* h) {
   if (!h) return SIM_OK;
   cudaStreamSynchronize(h->stream);
-  void* ptrs[] = {h->p, h->g, h->m, h->v, h->w1b, h->w2b, h->loss, h->err};
-  for (void* p : ptrs) if (p) cudaFree(p);
+  if (h->mem) cudaFree(h->mem);
   delete h;
   return SIM_OK;
 }

@@ -35,11 +35,23 @@ __device__ __forceinline__ uint64_t make_sdesc(uint32_t saddr, uint32_t lbo, uin
   return d;
 }
 
-// Instruction descriptor of kind::f16 with BF16 A and B, FP32 accumulator, both K-major.
-__host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N) {
+// The transpose of a K-major tile (above) as an operand: the tile of matrix T [k][n] read
+// MN-major, its rows k the reduction dimension, from the 16-row step that starts at saddr.
+// A core matrix of the tile (8 rows x 16 bytes along n) is one of the MN-major layout too;
+// 8-element groups along n are 128 bytes apart (the stride offset), 8-row groups along k
+// `rows8` bytes (the leading offset).
+__device__ __forceinline__ uint64_t mn_desc(uint32_t saddr, uint32_t rows8) {
+  return make_sdesc(saddr, rows8, 128);
+}
+
+// Instruction descriptor of kind::f16 with BF16 A and B, FP32 accumulator; each operand
+// K-major, or MN-major where the flag says so.
+__host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N, bool a_mn = false, bool b_mn = false) {
   return (1u << 4)                       // D format: F32
          | (1u << 7)                     // A format: BF16
          | (1u << 10)                    // B format: BF16
+         | ((a_mn ? 1u : 0u) << 15)      // A major
+         | ((b_mn ? 1u : 0u) << 16)      // B major
          | ((uint32_t)(N >> 3) << 17)    // N / 8
          | ((uint32_t)(M >> 4) << 24);   // M / 16
 }

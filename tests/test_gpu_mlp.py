@@ -385,3 +385,25 @@ def test_bounded_tensor_core_wait_times_out_and_leaves_the_device_usable():
     y = mlp(p).forward(to_dev(f)).cpu().numpy()
     ref = oracle.mlp_forward(p, M.bf16(f))
     assert np.abs(y - ref).max() <= 5e-3 * max(np.abs(ref).mean() + 1e-3, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("rows", [1, 128, 129, 152 * 128 + 1, 40001])
+def test_gradient_at_tile_and_grid_edges(rows):
+    """One row, whole and ragged tiles, one tile more than a block per SM, several tiles per
+    block (accumulated across tiles in tensor memory); the blocks' shares are added in a
+    fixed order, so a second run gives the same bits."""
+    p = M.init_params(8)
+    f = feats(rows, rows + 1)
+    t = np.random.default_rng(rows).normal(size=rows)
+    net, fd = mlp(p), to_dev(f)
+    td = torch.tensor(t, dtype=torch.float32, device="cuda")
+    L, g = net.grad(fd, td, 1.0 / rows)
+    L2, g2 = net.grad(fd, td, 1.0 / rows)
+    assert L == L2 and torch.equal(g, g2)
+    L_ref, g_ref = M.loss_and_grad(p, M.bf16(f), t, 1.0 / rows, bf16_ops=True)
+    assert L == pytest.approx(L_ref, rel=1e-2)
+    o, g = 0, g.cpu().numpy()
+    for name, shape in M.SIZES:
+        n = int(np.prod(shape))
+        assert np.abs(g[o:o + n] - g_ref[o:o + n]).max() <= 2e-2 * np.abs(g_ref[o:o + n]).max() + 1e-7, name
+        o += n
