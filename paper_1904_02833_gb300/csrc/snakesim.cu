@@ -1209,8 +1209,7 @@ SimStatus sim_calib_backward(SimHandle* h, const float* tips_bar, float* grad_th
   if (!h || !tips_bar || !grad_theta) return fail(SIM_EINVAL, "null handle or buffer");
   if (!h->calib) return fail(SIM_EINVAL, "no calibration forward pass to differentiate");
   std::string err;
-  SimStatus st = calib_backward(*h->calib, h->prm, h->node_off_d, h->link_off_d, tips_bar, grad_theta,
-                                h->stream, err);
+  SimStatus st = calib_backward(*h->calib, h->prm, tips_bar, grad_theta, h->stream, err);
   if (st != SIM_OK) return fail(st, err);
   return SIM_OK;
 }

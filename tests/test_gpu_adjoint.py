@@ -133,3 +133,35 @@ def test_calibration_batch_runs_and_matches_oracle_on_samples():
     for k in range(5):
         scale = np.abs(g_o[:, k]).max()
         assert np.abs(g[sel, k] - g_o[:, k]).max() <= 2e-2 * scale, (k, g[sel, k], g_o[:, k])
+
+
+@pytest.mark.parametrize("iters", [3, 14])
+def test_gradient_at_warp_edges_and_off_chip_iterates(iters):
+    """Snakes of 2, 32, 33, 64, 65 and 128 nodes in one batch (a thread per node: ends of
+    warps, blocks sized for the longest), the iterates of a substep on chip (3 updates) and
+    in the global scratch (14 updates of 128 nodes), against the oracle's dual-number
+    gradient; a second backward pass over the same rollout gives the same bits."""
+    from paper_1904_02833_gb300.calib import rollout, theta_of
+    from paper_1904_02833_gb300.sim import SnakeSim
+    steps = 3
+    truth, guess = W.calibration(n=6, seed=9)
+    for w in (truth, guess):
+        w["n_links"][:] = [1, 1, 4, 7, 8, 1]
+        w["seg_per_link"][:] = [1, 31, 8, 9, 8, 127]
+    assert W.n_nodes(guess).tolist() == [2, 32, 33, 64, 65, 128]
+    s = W.solver_settings(iters=iters)
+    ot = oracle.OracleSim(truth, s)
+    target = ot.step(steps, tip=True)
+    sim = SnakeSim(guess, s)
+    th = theta_of(guess).cuda().requires_grad_(True)
+    tips = rollout(sim, th, steps, 2)
+    tg = torch.tensor(target, dtype=torch.float32, device="cuda")
+    loss = ((tips - tg) ** 2).sum(-1).mean(0).sum()
+    g, = torch.autograd.grad(loss, th, retain_graph=True)
+    g2, = torch.autograd.grad(loss, th)
+    assert torch.equal(g, g2)
+    g = g.cpu().numpy()
+    og = oracle.OracleSim(guess, s)
+    _, g_o = og.calib_grad(steps, target)
+    for k in range(5):
+        assert np.abs(g[:, k] - g_o[:, k]).max() <= 2e-2 * np.abs(g_o[:, k]).max(), (k, g[:, k], g_o[:, k])
