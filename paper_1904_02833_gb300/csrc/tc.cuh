@@ -120,6 +120,39 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// The same in two steps, N = 16 or 32 columns: the load, then the wait that makes its
+// registers valid (they pass through it, so no use of them can move before it).  One load
+// may be in flight while the values of another are worked on; the wait is for all of them.
+#define TC_R4(r, i) "+r"(r[i]), "+r"(r[i + 1]), "+r"(r[i + 2]), "+r"(r[i + 3])
+#define TC_O4(r, i) "=r"(r[i]), "=r"(r[i + 1]), "=r"(r[i + 2]), "=r"(r[i + 3])
+__device__ __forceinline__ void tmem_load(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      : TC_O4(r, 0), TC_O4(r, 4), TC_O4(r, 8), TC_O4(r, 12), TC_O4(r, 16), TC_O4(r, 20), TC_O4(r, 24), TC_O4(r, 28)
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_load(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      : TC_O4(r, 0), TC_O4(r, 4), TC_O4(r, 8), TC_O4(r, 12)
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : TC_R4(r, 0), TC_R4(r, 4), TC_R4(r, 8), TC_R4(r, 12), TC_R4(r, 16), TC_R4(r, 20), TC_R4(r, 24),
+                 TC_R4(r, 28)::"memory");
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[16], uint32_t (&q)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : TC_R4(r, 0), TC_R4(r, 4), TC_R4(r, 8), TC_R4(r, 12), TC_R4(q, 0), TC_R4(q, 4), TC_R4(q, 8),
+                 TC_R4(q, 12)::"memory");
+}
+#undef TC_R4
+#undef TC_O4
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(mbar)), "r"(count)

@@ -407,3 +407,18 @@ def test_gradient_at_tile_and_grid_edges(rows):
         n = int(np.prod(shape))
         assert np.abs(g[o:o + n] - g_ref[o:o + n]).max() <= 2e-2 * np.abs(g_ref[o:o + n]).max() + 1e-7, name
         o += n
+
+
+@pytest.mark.parametrize("rows", [129, 304 * 128 + 1, 2 * 304 * 128 + 77, 5 * 304 * 128])
+def test_forward_does_not_depend_on_the_tile_schedule(rows):
+    """A row's output is the same bits whichever block, group and turn takes its tile: one
+    tile more than the blocks, more than both groups of every block, several turns, against
+    the same rows in calls of one tile each (sampled)."""
+    p = M.init_params(10)
+    f = feats(rows, 5)
+    net, fd = mlp(p), to_dev(f)
+    y = net.forward(fd)
+    for t0 in sorted({0, 128, (rows // 256) * 128, (rows - 1) // 128 * 128}):
+        t1 = min(rows, t0 + 128)
+        one = net.forward(fd[t0:t1].contiguous())
+        assert torch.equal(one, y[t0:t1]), t0
