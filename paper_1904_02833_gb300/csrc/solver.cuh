@@ -60,10 +60,23 @@ __device__ __forceinline__ float atan_unit(float t) {
   p = fmaf(p, s, 9.999998808e-01f);
   return t * p;
 }
+// 1 / a for 1 < a: the hardware's approximate reciprocal and one Newton step (rounded like
+// the exact value unless that lies within ~2^-45 of a rounding boundary), without the
+// branches of the general correctly rounded reciprocal, which every pass would issue for
+// the rare steep angles.
+__device__ __forceinline__ float rcp_approx(float a) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a));
+  return y;
+}
+__device__ __forceinline__ float rcp_newton(float a) {
+  const float y = rcp_approx(a);
+  return fmaf(fmaf(-a, y, 1.f), y, y);
+}
 __device__ __forceinline__ float atan_any(float t) {
   const float a = fabsf(t);
   const bool big = a > 1.f;
-  const float p = atan_unit(big ? __frcp_rn(a) : a);
+  const float p = atan_unit(big ? rcp_newton(a) : a);
   return copysignf(big ? 1.57079632679489662f - p : p, t);
 }
 // atan2(y, x) for the bend angles from the same polynomial, without branches: atan(y / x),
@@ -125,6 +138,13 @@ struct SnakeK {
 // |p| <= mu ln, or with anisotropic friction (the wheels and scales of Sec. V) the ellipse
 // (p_t / mu)^2 + (p_s / mu_side)^2 <= ln^2 in the body frame (t = (bx, by) along the chain,
 // s = z x t), projected radially in the coordinates scaled by the two coefficients.
+// disc_scale is the disc's factor alone.
+__device__ __forceinline__ float disc_scale(const SnakeK& S, float ln, float px, float py) {
+  // scale 1 inside the disc, rad / |p| outside, 0 for an empty disc; no branches
+  const float rad = S.mu * ln;
+  const float n2 = px * px + py * py;
+  return (n2 > rad * rad) ? (rad > 0.f ? rad * rsqrtf(n2) : 0.f) : 1.f;
+}
 template <bool ANISO>
 __device__ __forceinline__ void friction_limit(const SnakeK& S, float bx, float by, float ln, float& px,
                                                float& py) {
@@ -137,10 +157,7 @@ __device__ __forceinline__ void friction_limit(const SnakeK& S, float bx, float 
     px = a * bx - b * by;
     py = a * by + b * bx;
   } else {
-    // scale 1 inside the disc, rad / |p| outside, 0 for an empty disc; no branches
-    const float rad = S.mu * ln;
-    const float n2 = px * px + py * py;
-    const float sc = (n2 > rad * rad) ? (rad > 0.f ? rad * rsqrtf(n2) : 0.f) : 1.f;
+    const float sc = disc_scale(S, ln, px, py);
     px *= sc; py *= sc;
   }
 }
@@ -151,23 +168,15 @@ __device__ __forceinline__ void friction_limit(const SnakeK& S, float bx, float 
 
 namespace snakesim {
 
-// One pass over the rows at the current positions and multipliers.
-//   WARM = false: Jacobi pass.  Evaluates every row at (x^k, lambda^k), returns the
-//     group's normalised residual, and (unless `stop` comes back true) replaces lambda by
-//     its relaxed update and moves every free node by w_i sum_j grad_i c_j d_j.
-//   WARM = true: warm-start pass.  Uses d_j = lambda_j (zeroing rows that do not exist
-//     or touch no free node) and applies it, so that M (x - x~) = J^T lambda.
-// `stop` returns the group's stop decision (residual <= tol or cap reached).
-// The pass has no branches on row existence: every row of every node slot is evaluated
-// (on a straight dummy segment where the segment does not exist) and a row that does not
-// exist contributes d = 0 and residual 0, so that the lane's node slots form independent
-// instruction streams the scheduler can interleave.
-template <int NPL, int G, bool WARM, bool ANISO>
-__device__ __forceinline__ float row_pass(const SnakeK& S, const SolverArgs& A, int q,
-                                          bool live, int kiter, const float (&xs)[NPL][3],
-                                          float (&dx)[NPL][3], const float (&xsl)[3],
-                                          const float (&xsr)[3], float (&lam)[NPL][6],
-                                          const float (&th)[NPL], bool& stop) {
+// Warm-start pass at the predicted positions: uses d_j = lambda_j (zeroing rows that do not
+// exist or touch no free node) and applies it, so that M (x - x~) = J^T lambda.
+// No branches on row existence: every row of every node slot is evaluated (on a straight
+// dummy segment where the segment does not exist) and a row that does not exist contributes
+// d = 0, so that the lane's node slots form independent instruction streams.
+template <int NPL, int G>
+__device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, int q, bool live,
+                                          const float (&xs)[NPL][3], float (&dx)[NPL][3], const float (&xsl)[3],
+                                          const float (&xsr)[3], float (&lam)[NPL][6]) {
   const float L0 = S.L0;
   // neighbour displacements across the lane boundary
   float dxl[3], dxr[3];
@@ -192,11 +201,9 @@ __device__ __forceinline__ float row_pass(const SnakeK& S, const SolverArgs& A, 
     return make_seg(on ? ex : 1.f, on ? ey : 0.f, on ? ez : 0.f, L0);
   };
   float acc[NPL][3];
-  float dl[NPL][6];
   float accL[3] = {0.f, 0.f, 0.f}, accR[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int j = 0; j < NPL; ++j) acc[j][0] = acc[j][1] = acc[j][2] = 0.f;
-  float r = 0.f, q2 = 0.f;
   Seg sp = seg(0);  // segment i0 - 1
 #pragma unroll
   for (int j = 0; j < NPL; ++j) {
@@ -208,107 +215,244 @@ __device__ __forceinline__ float row_pass(const SnakeK& S, const SolverArgs& A, 
     const float wr = (i + 1 < S.nfix) ? 0.f : S.inv_m;
     float* tl = (j > 0) ? acc[j - 1] : accL;          // node i-1
     float* tr = (j + 1 < NPL) ? acc[j + 1] : accR;    // node i+1
-    // ---- stretch (i, i+1): c = |e| - L0 (Eq. 3 with a constant rest length)
     {
-      const float c = sc.len - L0;
-      const float wg = wi + wr;
-      const bool on = act && i + 1 <= S.N - 1 && wg > 0.f;
-      float d;
-      if (WARM) d = lam[j][0];
-      else {
-        const float l = lam[j][0];
-        r = fmaxf(r, on ? fabsf(c + S.at_s * l) : 0.f);
-        d = __fdividef(A.omega * (-c - S.at_s * l), wg + S.at_s);
-      }
-      d = on ? d : 0.f;
-      dl[j][0] = d;
+      const float d = act && i + 1 <= S.N - 1 && wi + wr > 0.f ? lam[j][0] : 0.f;
+      lam[j][0] = d;
       acc[j][0] -= sc.nx * d; acc[j][1] -= sc.ny * d; acc[j][2] -= sc.nz * d;
       tr[0] += sc.nx * d; tr[1] += sc.ny * d; tr[2] += sc.nz * d;
     }
-    // ---- yaw and pitch bend centred on node i (rows in length units: L0 x angle)
     const bool bend = act && i >= 1 && i <= S.N - 2;
-    // yaw: L0 (atan2(z . (e1 x e2), e1_h . e2_h) - theta_rest)
     {
-      const float cz = sp.ex * sc.ey - sp.ey * sc.ex;
-      const float dh = sp.ex * sc.ex + sp.ey * sc.ey;
-      const float c = L0 * (atan2_bend(cz, dh) - th[j]);
       const float g0x = sp.gyx, g0y = sp.gyy;                     // node i-1
       const float g1x = -sp.gyx - sc.gyx, g1y = -sp.gyy - sc.gyy; // node i
       const float g2x = sc.gyx, g2y = sc.gyy;                     // node i+1
       const float wg = wl * (g0x * g0x + g0y * g0y) + wi * (g1x * g1x + g1y * g1y) +
                        wr * (g2x * g2x + g2y * g2y);
-      const bool on = bend && wg > 0.f;
-      float d;
-      if (WARM) d = lam[j][1];
-      else {
-        const float l = lam[j][1];
-        r = fmaxf(r, on ? fabsf(c + S.at_b * l) : 0.f);
-        d = __fdividef(A.omega * (-c - S.at_b * l), wg + S.at_b);
-      }
-      d = on ? d : 0.f;
-      dl[j][1] = d;
+      const float d = bend && wg > 0.f ? lam[j][1] : 0.f;
+      lam[j][1] = d;
       tl[0] += g0x * d; tl[1] += g0y * d;
       acc[j][0] += g1x * d; acc[j][1] += g1y * d;
       tr[0] += g2x * d; tr[1] += g2y * d;
     }
-    // pitch: L0 (elevation(e2) - elevation(e1))
     {
-      const float c = L0 * (sc.beta - sp.beta);
       const float g0x = sp.gpx, g0y = sp.gpy, g0z = sp.gpz;
       const float g1x = -sp.gpx - sc.gpx, g1y = -sp.gpy - sc.gpy, g1z = -sp.gpz - sc.gpz;
       const float g2x = sc.gpx, g2y = sc.gpy, g2z = sc.gpz;
       const float wg = wl * (g0x * g0x + g0y * g0y + g0z * g0z) +
                        wi * (g1x * g1x + g1y * g1y + g1z * g1z) +
                        wr * (g2x * g2x + g2y * g2y + g2z * g2z);
-      const bool on = bend && wg > 0.f;
-      float d;
-      if (WARM) d = lam[j][2];
-      else {
-        const float l = lam[j][2];
-        r = fmaxf(r, on ? fabsf(c + S.at_b * l) : 0.f);
-        d = __fdividef(A.omega * (-c - S.at_b * l), wg + S.at_b);
-      }
-      d = on ? d : 0.f;
-      dl[j][2] = d;
+      const float d = bend && wg > 0.f ? lam[j][2] : 0.f;
+      lam[j][2] = d;
       tl[0] += g0x * d; tl[1] += g0y * d; tl[2] += g0z * d;
       acc[j][0] += g1x * d; acc[j][1] += g1y * d; acc[j][2] += g1z * d;
       tr[0] += g2x * d; tr[1] += g2y * d; tr[2] += g2z * d;
     }
     sp = sc;
   }
-  // ---- ground contact (Eq. 7, z - r >= 0) and Coulomb friction pair of every node slot.
-  // Their residual terms decide nothing in a pass where every group's bilateral terms
-  // already exceed the tolerance (the group cannot stop) and the cap is not reached, so
-  // they are evaluated only when some group's could decide it (warp-uniform choice
-  // between two compiled forms of the loop); the updates are the same either way.
-  auto contact_rows = [&](auto with_residual) {
-    constexpr bool RES = decltype(with_residual)::value;
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    const int i = i0 + j;
+    const bool on = live && i < S.N && A.contact && i >= S.nfix;
+#pragma unroll
+    for (int k = 3; k < 6; ++k) lam[j][k] = on ? lam[j][k] : 0.f;
+    acc[j][2] += lam[j][3];
+    acc[j][0] += lam[j][4];
+    acc[j][1] += lam[j][5];
+  }
+  // contributions that cross lane boundaries
+  float fromR[3], fromL[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    fromR[d] = __shfl_down_sync(kFull, accL[d], 1, G);  // right lane's rows -> my last node
+    fromL[d] = __shfl_up_sync(kFull, accR[d], 1, G);    // left lane's rows -> my first node
+  }
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    const int i = i0 + j;
+    float ax = acc[j][0], ay = acc[j][1], az = acc[j][2];
+    if (j == 0 && q > 0) { ax += fromL[0]; ay += fromL[1]; az += fromL[2]; }
+    if (j == NPL - 1 && q < G - 1) { ax += fromR[0]; ay += fromR[1]; az += fromR[2]; }
+    const bool on = live && i < S.N;
+    const float wi = (i < S.nfix) ? 0.f : S.inv_m;
+    dx[j][0] = on ? dx[j][0] + wi * ax : dx[j][0];
+    dx[j][1] = on ? dx[j][1] + wi * ay : dx[j][1];
+    dx[j][2] = on ? dx[j][2] + wi * az : dx[j][2];
+  }
+}
+
+// Jacobi iterations of one substep: pass k evaluates every row at (x^k, lambda^k) and, unless
+// the group's normalised residual is within the tolerance or k is the cap, replaces lambda by
+// its relaxed update and moves every free node by w_i sum_j grad_i c_j d_j.  Returns the
+// residual at the final iterate and the updates applied.
+//
+// What bounds it: the issue slots and latency of a warp's own pass (a snake's passes are a
+// serial chain, and in a tolerance run the slowest snake's chain is the launch's length), so
+// the pass carries nothing that does not change from pass to pass:
+//  * substep-start differences, contact heights and the friction frame are formed once;
+//  * a row that does not exist has a zero in the constant its update is multiplied by (the
+//    stretch row's reciprocal weight, the contact and friction rows' omega m, an infinite
+//    bend weight) instead of selects; its segment is a straight dummy whose positions are
+//    chosen once.  Residual terms are masked by a 0 / 1 factor;
+//  * a pass in which every live group has a bilateral term over the tolerance (and the cap
+//    is not reached) stops nothing: it needs neither the contact and friction residuals nor
+//    the stop logic, and updates without selects.  The other passes take the second form.
+// Measured against row selects, the general reciprocal and the residuals of every pass in one
+// form, same bits: one 41-node snake at ten updates 256 -> 200 us per env-step, 4096 uneven
+// snakes 785 -> 600 us; 8192 snakes to 1e-4 cold 49-58 -> 32-35 ms, 256 cantilevers to 1e-6
+// 30.9 -> 18.8 ms.
+template <int NPL, int G, bool ANISO>
+__device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int q, bool valid,
+                                       const float (&xs)[NPL][3], float (&dx)[NPL][3], const float (&xsl)[3],
+                                       const float (&xsr)[3], float (&lam)[NPL][6], const float (&th)[NPL],
+                                       float& r_end, int& updates) {
+  const float L0 = S.L0;
+  const int i0 = q * NPL;
+  const unsigned lane = threadIdx.x & 31u;
+  const unsigned gm = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(unsigned)(G - 1)));
+  // constants of the substep
+  float xd[NPL + 1][3];         // segment vectors at the substep start, u: segment i0 + u - 1
+  float w[NPL + 2];             // inverse masses of nodes i0 - 1 .. i0 + NPL
+  float ws[NPL], rs[NPL];       // stretch: residual mask, omega-free reciprocal weight
+  float wb[NPL], ab[NPL];       // bend: residual mask, compliance in the weight (inf: no row)
+  float zc[NPL], om[NPL];       // contact: height above the radius, omega m (0: no row)
+  float tx0[ANISO ? NPL : 1], ty0[ANISO ? NPL : 1];  // body tangent (anisotropic friction)
+#pragma unroll
+  for (int u = 0; u <= NPL; ++u) {
+    const int i = i0 + u - 1;
+    const bool on = valid && i >= 0 && i + 1 <= S.N - 1;
+    const float* a = (u == 0) ? xsl : xs[u > 0 ? u - 1 : 0];
+    const float* b = (u == NPL) ? xsr : xs[u < NPL ? u : 0];
+    xd[u][0] = on ? b[0] - a[0] : 1.f;
+    xd[u][1] = on ? b[1] - a[1] : 0.f;
+    xd[u][2] = on ? b[2] - a[2] : 0.f;
+  }
+#pragma unroll
+  for (int u = 0; u < NPL + 2; ++u) {
+    const int i = i0 + u - 1;
+    w[u] = valid && i >= S.nfix && i < S.N ? S.inv_m : 0.f;
+  }
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    const int i = i0 + j;
+    const float wg = w[j + 1] + w[j + 2];
+    const bool st = valid && i + 1 <= S.N - 1 && wg > 0.f;
+    const bool bd = valid && i >= 1 && i <= S.N - 2 && (w[j] + w[j + 1] + w[j + 2] > 0.f);
+    ws[j] = st ? 1.f : 0.f;
+    rs[j] = st ? rcp_approx(wg + S.at_s) : 0.f;
+    wb[j] = bd ? 1.f : 0.f;
+    ab[j] = bd ? S.at_b : INFINITY;
+    zc[j] = xs[j][2] - S.radius;
+    om[j] = A.contact && w[j + 1] > 0.f ? S.om_m : 0.f;
+    if constexpr (ANISO) {
+      // body tangent at the substep start
+      tx0[j] = 1.f; ty0[j] = 0.f;
+      if (S.mu_side > 0.f) {
+        float ax0 = xs[j][0], ay0 = xs[j][1], bx0 = xs[j][0], by0 = xs[j][1];
+        if (i >= 1) { ax0 = (j > 0) ? xs[j - 1][0] : xsl[0]; ay0 = (j > 0) ? xs[j - 1][1] : xsl[1]; }
+        if (i + 1 <= S.N - 1) {
+          bx0 = (j + 1 < NPL) ? xs[j + 1][0] : xsr[0];
+          by0 = (j + 1 < NPL) ? xs[j + 1][1] : xsr[1];
+        }
+        const float ex = bx0 - ax0, ey = by0 - ay0, en2 = ex * ex + ey * ey;
+        if (en2 > 0.f) { const float ie = rsqrtf(en2); tx0[j] = ex * ie; ty0[j] = ey * ie; }
+      }
+    }
+  }
+  bool live = valid;
+  r_end = 0.f;
+  updates = 0;
+  for (int k = 0;; ++k) {
+    // neighbour displacements across the lane boundary
+    float dxl[3], dxr[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      dxl[d] = __shfl_up_sync(kFull, dx[NPL - 1][d], 1, G);
+      dxr[d] = __shfl_down_sync(kFull, dx[0][d], 1, G);
+    }
+    auto seg = [&](int u) {
+      const float* ad = (u == 0) ? dxl : dx[u > 0 ? u - 1 : 0];
+      const float* bd = (u == NPL) ? dxr : dx[u < NPL ? u : 0];
+      return make_seg(xd[u][0] + (bd[0] - ad[0]), xd[u][1] + (bd[1] - ad[1]), xd[u][2] + (bd[2] - ad[2]), L0);
+    };
+    float acc[NPL][3], dl[NPL][6];
+    float accL[3] = {0.f, 0.f, 0.f}, accR[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) acc[j][0] = acc[j][1] = acc[j][2] = 0.f;
+    float r = 0.f;
+    Seg sp = seg(0);  // segment i0 - 1
 #pragma unroll
     for (int j = 0; j < NPL; ++j) {
-      const int i = i0 + j;
-      const bool act = live && i < S.N;
-      const float wi = (i < S.nfix) ? 0.f : S.inv_m;
-      const bool on = act && A.contact && wi > 0.f;
-      const float ln = lam[j][3];
-      const float cn = (xs[j][2] - S.radius) + dx[j][2];
-      const float ux = dx[j][0], uy = dx[j][1];
-      float dn, fx, fy;
-      if (WARM) { dn = ln; fx = lam[j][4]; fy = lam[j][5]; }
-      else {
-        // body tangent at the substep start (anisotropic friction only)
-        float bx = 1.f, by = 0.f;
-        if (ANISO && S.mu_side > 0.f) {
-          float ax0 = xs[j][0], ay0 = xs[j][1], bx0 = xs[j][0], by0 = xs[j][1];
-          if (i >= 1) { ax0 = (j > 0) ? xs[j - 1][0] : xsl[0]; ay0 = (j > 0) ? xs[j - 1][1] : xsl[1]; }
-          if (i + 1 <= S.N - 1) {
-            bx0 = (j + 1 < NPL) ? xs[j + 1][0] : xsr[0];
-            by0 = (j + 1 < NPL) ? xs[j + 1][1] : xsr[1];
-          }
-          const float ex = bx0 - ax0, ey = by0 - ay0, en2 = ex * ex + ey * ey;
-          if (en2 > 0.f) { const float ie = rsqrtf(en2); bx = ex * ie; by = ey * ie; }
-        }
+      const Seg sc = seg(j + 1);  // segment i
+      const float wl = w[j], wi = w[j + 1], wr = w[j + 2];
+      float* tl = (j > 0) ? acc[j - 1] : accL;        // node i-1
+      float* tr = (j + 1 < NPL) ? acc[j + 1] : accR;  // node i+1
+      // ---- stretch (i, i+1): c = |e| - L0 (Eq. 3 with a constant rest length)
+      {
+        const float c = sc.len - L0;
+        const float l = lam[j][0];
+        r = fmaxf(r, fabsf(c + S.at_s * l) * ws[j]);
+        const float d = __fmul_rn(A.omega * (-c - S.at_s * l), rs[j]);
+        dl[j][0] = d;
+        acc[j][0] -= sc.nx * d; acc[j][1] -= sc.ny * d; acc[j][2] -= sc.nz * d;
+        tr[0] += sc.nx * d; tr[1] += sc.ny * d; tr[2] += sc.nz * d;
+      }
+      // ---- yaw and pitch bend centred on node i (rows in length units: L0 x angle)
+      // yaw: L0 (atan2(z . (e1 x e2), e1_h . e2_h) - theta_rest)
+      {
+        const float cz = sp.ex * sc.ey - sp.ey * sc.ex;
+        const float dh = sp.ex * sc.ex + sp.ey * sc.ey;
+        const float c = L0 * (atan2_bend(cz, dh) - th[j]);
+        const float g0x = sp.gyx, g0y = sp.gyy;                     // node i-1
+        const float g1x = -sp.gyx - sc.gyx, g1y = -sp.gyy - sc.gyy; // node i
+        const float g2x = sc.gyx, g2y = sc.gyy;                     // node i+1
+        const float wg = wl * (g0x * g0x + g0y * g0y) + wi * (g1x * g1x + g1y * g1y) +
+                         wr * (g2x * g2x + g2y * g2y);
+        const float l = lam[j][1];
+        r = fmaxf(r, fabsf(c + S.at_b * l) * wb[j]);
+        const float d = __fmul_rn(A.omega * (-c - S.at_b * l), rcp_approx(wg + ab[j]));
+        dl[j][1] = d;
+        tl[0] += g0x * d; tl[1] += g0y * d;
+        acc[j][0] += g1x * d; acc[j][1] += g1y * d;
+        tr[0] += g2x * d; tr[1] += g2y * d;
+      }
+      // pitch: L0 (elevation(e2) - elevation(e1))
+      {
+        const float c = L0 * (sc.beta - sp.beta);
+        const float g0x = sp.gpx, g0y = sp.gpy, g0z = sp.gpz;
+        const float g1x = -sp.gpx - sc.gpx, g1y = -sp.gpy - sc.gpy, g1z = -sp.gpz - sc.gpz;
+        const float g2x = sc.gpx, g2y = sc.gpy, g2z = sc.gpz;
+        const float wg = wl * (g0x * g0x + g0y * g0y + g0z * g0z) +
+                         wi * (g1x * g1x + g1y * g1y + g1z * g1z) +
+                         wr * (g2x * g2x + g2y * g2y + g2z * g2z);
+        const float l = lam[j][2];
+        r = fmaxf(r, fabsf(c + S.at_b * l) * wb[j]);
+        const float d = __fmul_rn(A.omega * (-c - S.at_b * l), rcp_approx(wg + ab[j]));
+        dl[j][2] = d;
+        tl[0] += g0x * d; tl[1] += g0y * d; tl[2] += g0z * d;
+        acc[j][0] += g1x * d; acc[j][1] += g1y * d; acc[j][2] += g1z * d;
+        tr[0] += g2x * d; tr[1] += g2y * d; tr[2] += g2z * d;
+      }
+      sp = sc;
+    }
+    // a group could stop only if none of its lanes has a bilateral term over the tolerance
+    // (a non-finite term counts as not over, so that it reaches the residual)
+    const unsigned over_b = __ballot_sync(kFull, r * S.inv_L0 > A.tol);
+    const bool may_stop = __any_sync(kFull, live && (over_b & gm) == 0u) || k >= A.K;
+    // ---- ground contact (Eq. 7, z - r >= 0) and Coulomb friction pair of every node slot,
+    // the stop decision (RES) and the update; returns true when every group has stopped
+    auto finish = [&](auto res) -> bool {
+      constexpr bool RES = decltype(res)::value;
+      float q2 = 0.f;
+#pragma unroll
+      for (int j = 0; j < NPL; ++j) {
+        const float ln = lam[j][3];
+        const float cn = zc[j] + dx[j][2];
+        const float ux = dx[j][0], uy = dx[j][1];
+        const float bx = ANISO ? tx0[ANISO ? j : 0] : 1.f, by = ANISO ? ty0[ANISO ? j : 0] : 0.f;
         if constexpr (RES) {
           // residuals: Fischer-Burmeister on (c_n, w lambda_n); natural map of the cone
+          const float wi = w[j + 1];
+          const bool on = om[j] > 0.f;
           const float b = wi * ln;
           r = fmaxf(r, on ? fabsf(cn + b - sqrtf(cn * cn + b * b)) : 0.f);
           const float ax = wi * lam[j][4], ay = wi * lam[j][5];
@@ -318,72 +462,72 @@ __device__ __forceinline__ float row_pass(const SnakeK& S, const SolverArgs& A, 
           q2 = fmaxf(q2, on ? (ax - px) * (ax - px) + (ay - py) * (ay - py) : 0.f);
         }
         // contact: lambda_n <- max(0, lambda_n + omega (-c_n / w))
-        const float nl = fmaxf(0.f, ln - S.om_m * cn);
-        dn = nl - ln;
+        const float nl = fmaxf(0.f, ln - om[j] * cn);
+        const float dn = nl - ln;
         // friction: relaxed update limited to the Coulomb set of the current iterate's
         // lambda_n
-        float tx = lam[j][4] - S.om_m * ux;
-        float ty = lam[j][5] - S.om_m * uy;
-        friction_limit<ANISO>(S, bx, by, ln, tx, ty);
-        fx = tx - lam[j][4]; fy = ty - lam[j][5];
+        float tx = lam[j][4] - om[j] * ux;
+        float ty = lam[j][5] - om[j] * uy;
+        float fx, fy;
+        if constexpr (ANISO) {
+          friction_limit<ANISO>(S, bx, by, ln, tx, ty);
+          fx = tx - lam[j][4]; fy = ty - lam[j][5];
+        } else {
+          const float sc = disc_scale(S, ln, tx, ty);
+          fx = fmaf(tx, sc, -lam[j][4]); fy = fmaf(ty, sc, -lam[j][5]);
+        }
+        dl[j][3] = dn; dl[j][4] = fx; dl[j][5] = fy;
+        acc[j][2] += dn;
+        acc[j][0] += fx;
+        acc[j][1] += fy;
       }
-      dn = on ? dn : 0.f; fx = on ? fx : 0.f; fy = on ? fy : 0.f;
-      dl[j][3] = dn; dl[j][4] = fx; dl[j][5] = fy;
-      acc[j][2] += dn;
-      acc[j][0] += fx;
-      acc[j][1] += fy;
+      if constexpr (RES) {
+        // every term is a length: one scaling by 1 / L0 (monotone, so the max is the same)
+        r = fmaxf(r, sqrtf(q2)) * S.inv_L0;
+        if (!(r <= 3.0e38f)) r = INFINITY;  // NaN -> inf so that the max keeps it
+        // one ballot decides every group's stop; the group's max residual is reduced only in
+        // the (rare) passes where some live group stops, to be recorded
+        const unsigned over = __ballot_sync(kFull, !(r <= A.tol));
+        const bool stop = ((over & gm) == 0u) || (k >= A.K);
+        if (__any_sync(kFull, stop && live)) {
+          r = group_max<G>(r);
+          if (stop && live) {
+            live = false;
+            r_end = r;
+            updates = k;
+          }
+        }
+        if (__all_sync(kFull, !live)) return true;
+      }
+      // contributions that cross lane boundaries
+      float fromR[3], fromL[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        fromR[d] = __shfl_down_sync(kFull, accL[d], 1, G);  // right lane's rows -> my last node
+        fromL[d] = __shfl_up_sync(kFull, accR[d], 1, G);    // left lane's rows -> my first node
+      }
+#pragma unroll
+      for (int j = 0; j < NPL; ++j) {
+        float ax = acc[j][0], ay = acc[j][1], az = acc[j][2];
+        if (j == 0 && q > 0) { ax += fromL[0]; ay += fromL[1]; az += fromL[2]; }
+        if (j == NPL - 1 && q < G - 1) { ax += fromR[0]; ay += fromR[1]; az += fromR[2]; }
+        const float wi = w[j + 1];
+        if (G == 32 || live) {  // a group that has stopped keeps its state
+          dx[j][0] = dx[j][0] + wi * ax;
+          dx[j][1] = dx[j][1] + wi * ay;
+          dx[j][2] = dx[j][2] + wi * az;
+#pragma unroll
+          for (int m = 0; m < 6; ++m) lam[j][m] = lam[j][m] + dl[j][m];
+        }
+      }
+      return false;
+    };
+    if (may_stop) {
+      if (finish(std::true_type{})) break;
+    } else {
+      finish(std::false_type{});
     }
-  };
-  bool cf_residual = true;
-  if (!WARM) {
-    // a group could stop only if none of its lanes has a bilateral term over the
-    // tolerance (a non-finite term counts as not over, so that it reaches the residual)
-    const float rb = r * S.inv_L0;
-    const unsigned ln_ = threadIdx.x & 31u;
-    const unsigned gm = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (ln_ & ~(unsigned)(G - 1)));
-    const unsigned over_b = __ballot_sync(kFull, rb > A.tol);
-    cf_residual = __any_sync(kFull, live && (over_b & gm) == 0u) || kiter >= A.K;
   }
-  if (cf_residual) contact_rows(std::true_type{});
-  else contact_rows(std::false_type{});
-  if (!WARM) {
-    // every term is a length: one scaling by 1 / L0 (monotone, so the max is the same)
-    r = fmaxf(r, sqrtf(q2)) * S.inv_L0;
-    if (!(r <= 3.0e38f)) r = INFINITY;  // NaN -> inf so that the max keeps it
-    // one ballot decides every group's stop; the group's max residual is reduced only in
-    // the (rare) passes where some live group stops, to be recorded
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned over = __ballot_sync(kFull, !(r <= A.tol));
-    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(unsigned)(G - 1)));
-    stop = ((over & gmask) == 0u) || (kiter >= A.K);
-    if (__any_sync(kFull, stop && live)) r = group_max<G>(r);
-  } else {
-    stop = false;
-  }
-  // contributions that cross lane boundaries
-  float fromR[3], fromL[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    fromR[d] = __shfl_down_sync(kFull, accL[d], 1, G);  // right lane's rows -> my last node
-    fromL[d] = __shfl_up_sync(kFull, accR[d], 1, G);    // left lane's rows -> my first node
-  }
-  // update, by selects: a node slot beyond the snake or a group that stops keeps its state
-  const bool upd = live && !stop;
-#pragma unroll
-  for (int j = 0; j < NPL; ++j) {
-    const int i = i0 + j;
-    float ax = acc[j][0], ay = acc[j][1], az = acc[j][2];
-    if (j == 0 && q > 0) { ax += fromL[0]; ay += fromL[1]; az += fromL[2]; }
-    if (j == NPL - 1 && q < G - 1) { ax += fromR[0]; ay += fromR[1]; az += fromR[2]; }
-    const bool on = upd && i < S.N;
-    const float wi = (i < S.nfix) ? 0.f : S.inv_m;
-    dx[j][0] = on ? dx[j][0] + wi * ax : dx[j][0];
-    dx[j][1] = on ? dx[j][1] + wi * ay : dx[j][1];
-    dx[j][2] = on ? dx[j][2] + wi * az : dx[j][2];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) lam[j][k] = on ? (WARM ? dl[j][k] : lam[j][k] + dl[j][k]) : lam[j][k];
-  }
-  return r;
 }
 
 // Writes the 24 warm-start features (padded to 32, bf16) of the six rows each node owns,
@@ -787,7 +931,6 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid, float* sme
       xsl[d] = __shfl_up_sync(kFull, xs[NPL - 1][d], 1, G);
       xsr[d] = __shfl_down_sync(kFull, xs[0][d], 1, G);
     }
-    bool stop;
     if (A.warm == 0) {
 #pragma unroll
       for (int j = 0; j < NPL; ++j)
@@ -809,19 +952,14 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid, float* sme
           lam[j][k] = l;
         }
       }
-      row_pass<NPL, G, true, ANISO>(S, A, q, valid, 0, xs, dx, xsl, xsr, lam, th, stop);
+      warm_pass<NPL, G>(S, A, q, valid, xs, dx, xsl, xsr, lam);
     }
-    bool done = !valid;
     float rs = 0.f;
     int ks = 0;
     if (VAR == kVarPcr) {
       newton_pcr<NPL, G>(S, A, q, valid, xs, dx, lam, th, smem, rs, ks);
     } else {
-      for (int k = 0;; ++k) {
-        const float r = row_pass<NPL, G, false, ANISO>(S, A, q, !done, k, xs, dx, xsl, xsr, lam, th, stop);
-        if (!done && stop) { done = true; rs = r; ks = k; }
-        if (__all_sync(kFull, done)) break;
-      }
+      jacobi<NPL, G, ANISO>(S, A, q, valid, xs, dx, xsl, xsr, lam, th, rs, ks);
     }
     // a non-finite displacement anywhere in the snake marks the step (fmaxf drops NaN)
     float bad = 0.f;
