@@ -66,7 +66,9 @@ namespace {
 #endif
 // Persistent: every warp takes the next work item (32/G snakes of one node count) from
 // the layout's counter in global memory until none is left.
-template <int NPL, int G, bool SPLIT, int VAR>
+// WIDE (G = 32): the snakes of a layout with fewer lanes, one per warp, in that layout's
+// order of sums (see Roles in solver.cuh).
+template <int NPL, int G, bool SPLIT, int VAR, bool WIDE = false>
 __global__ void __launch_bounds__(128, SNAKE_MIN_BLOCKS) snake_solver_kernel(SolverArgs A) {
   extern __shared__ float solver_smem[];  // Newton + PCR only (kPcrFloatsPerSlot x 32 NPL per warp)
   const int lane = threadIdx.x & 31;
@@ -79,12 +81,13 @@ __global__ void __launch_bounds__(128, SNAKE_MIN_BLOCKS) snake_solver_kernel(Sol
     const int gi = lane / G;
     const bool ok = gi < item.y;
     const int snake = ok ? A.order[item.x + gi] : 0;
-    run_group<NPL, G, SPLIT, VAR>(A, snake, ok, solver_smem);
+    run_group<NPL, G, SPLIT, VAR, WIDE>(A, snake, ok, solver_smem);
   }
 }
 
 typedef void (*SolverKernel)(SolverArgs);
 constexpr int kLayouts = 12;
+
 // [split][solver variant: kVarJacobi, kVarAniso, kVarPcr][layout_id(G, NPL)]
 #define SNAKE_KERNELS(S, F)                                                                          \
   {snake_solver_kernel<1, 8, S, F>,  snake_solver_kernel<2, 8, S, F>,  snake_solver_kernel<3, 8, S, F>,  \
@@ -94,6 +97,12 @@ constexpr int kLayouts = 12;
 const SolverKernel kSolverKernels[2][3][kLayouts] = {
     {SNAKE_KERNELS(false, kVarJacobi), SNAKE_KERNELS(false, kVarAniso), SNAKE_KERNELS(false, kVarPcr)},
     {SNAKE_KERNELS(true, kVarJacobi), SNAKE_KERNELS(true, kVarAniso), SNAKE_KERNELS(true, kVarPcr)}};
+// [split][kVarJacobi, kVarAniso][nodes per lane - 1]
+const SolverKernel kWideKernels[2][2][2] = {
+    {{snake_solver_kernel<1, 32, false, kVarJacobi, true>, snake_solver_kernel<2, 32, false, kVarJacobi, true>},
+     {snake_solver_kernel<1, 32, false, kVarAniso, true>, snake_solver_kernel<2, 32, false, kVarAniso, true>}},
+    {{snake_solver_kernel<1, 32, true, kVarJacobi, true>, snake_solver_kernel<2, 32, true, kVarJacobi, true>},
+     {snake_solver_kernel<1, 32, true, kVarAniso, true>, snake_solver_kernel<2, 32, true, kVarAniso, true>}}};
 // dynamic shared memory of a block of the Newton + PCR kernels
 inline size_t pcr_smem_bytes(int lay) { return (size_t)4 * kPcrFloatsPerSlot * 32 * layout_npl(lay) * sizeof(float); }
 #undef SNAKE_KERNELS
@@ -237,7 +246,31 @@ __global__ void training_rows_kernel(const __nv_bfloat16* __restrict__ feat, con
 }
 
 // ------------------------------------------------------------------ handle
-struct SimHandle {
+// Work items of all snakes and what schedules and launches them.
+struct ItemSet {
+  int4* items = nullptr;
+  int* order = nullptr;
+  int n_items = 0;
+  // device scheduling (schedule_kernel): class of each snake, class offsets, scratch
+  int4* items0 = nullptr;
+  int *sched_cls = nullptr, *sched_base = nullptr, *sched_hist = nullptr, *sched_key = nullptr;
+  int n_cls = 0;
+  int lay_first[kLayouts + 1] = {};  // items of layout l are [lay_first[l], lay_first[l + 1])
+  int lay_grid[kLayouts] = {};
+  int lay_launch[kLayouts] = {};      // layouts with work, most work first
+  int n_lay = 0;
+  bool wide = false;                  // the 8- and 16-lane layouts run by WIDE kernels
+  void release() {
+    for (void* p : {(void*)items, (void*)items0, (void*)order, (void*)sched_cls, (void*)sched_base,
+                    (void*)sched_hist, (void*)sched_key})
+      if (p) cudaFree(p);
+    *this = ItemSet();
+  }
+};
+
+struct SimHandle : ItemSet {
+  ItemSet parked;  // the other choice of `wide`, once it has been built
+  int sms = 0;
   SimConfig cfg;
   int n = 0;
   long long n_nodes = 0, n_links = 0;
@@ -255,23 +288,12 @@ struct SimHandle {
   int *node_off_d = nullptr, *link_off_d = nullptr;
   float* resid = nullptr;
   int *iters = nullptr, *status = nullptr;
-  int4* items = nullptr;
-  int* order = nullptr;
-  int n_items = 0;
-  // device scheduling (schedule_kernel): class of each snake, class offsets, scratch
   // feature rows: the snakes of one layout take consecutive rows (network per layout);
   // snake s's rows start at 6 feat_off[s], layout l's nodes are [lay_fnode[l], lay_fnode[l+1])
   int* feat_off_d = nullptr;
   std::vector<int> feat_off;
   long long lay_fnode[kLayouts + 1] = {};
-  int4* items0 = nullptr;
-  int *sched_cls = nullptr, *sched_base = nullptr, *sched_hist = nullptr, *sched_key = nullptr;
-  int n_cls = 0;
-  int lay_first[kLayouts + 1] = {};  // items of layout l are [lay_first[l], lay_first[l + 1])
-  int lay_grid[kLayouts] = {};
-  int lay_launch[kLayouts] = {};      // layouts with work, most work first
   int aniso = 0;                      // some snake has anisotropic friction
-  int n_lay = 0;
   int* work = nullptr;                // [kLayouts] work-queue counters
   bool timing = false;                // record an event pair around every solver launch
   struct Timed { int lay; cudaEvent_t a, b; };
@@ -355,7 +377,30 @@ int solver_var(const SimHandle* h) {
   return h->aniso ? kVarAniso : kVarJacobi;
 }
 
+// Whether the snakes of the 8- and 16-lane layouts run one per warp, by the WIDE kernels (same
+// results).  A warp of several snakes shares its issue slots but walks three or four nodes
+// per lane and, to a tolerance, goes on until its slowest snake has converged.  Measured on
+// uneven snakes of 21-61 nodes (us per env-step, several per warp / one per warp): to 1e-4
+// from the previous multipliers 3245 / 1329 (one snake), 7004 / 2293 (1216), 10850 / 8045
+// (9728), 19724 / 14475 (19456), and alike from cold ones; at ten fixed updates 257 / 133
+// (one snake), 267 / 175 (1216), 334 / 339 (2432), 957 / 1047 (9728).  So: always to a
+// tolerance, and at fixed updates up to two snakes per warp slot of the chip.
+bool use_wide(const SimHandle* h) {
+  return solver_var(h) != kVarPcr && (h->cfg.tol > 0.f || h->n <= 16 * h->sms);
+}
+bool lay_wide(const SimHandle* h, int l) { return h->wide && layout_lanes(l) < 32; }
+
+// The kernel that runs the items of layout l.
+SolverKernel solver_kernel(const SimHandle* h, bool split, int l) {
+  const int var = solver_var(h);
+  if (lay_wide(h, l)) return kWideKernels[split ? 1 : 0][var][layout_lanes(l) * layout_npl(l) <= 32 ? 0 : 1];
+  return kSolverKernels[split ? 1 : 0][var][l];
+}
+
 SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = nullptr) {
+  // (autotuning times the layouts themselves)
+  static_cast<ItemSet*>(h)->release();
+  h->wide = !only_bucket && use_wide(h);
   // group snakes by node count, pack 32/G snakes per warp item, biggest work first;
   // `only_bucket` restricts the items to the node counts it lists (autotuning)
   std::map<int, std::vector<int>> buckets;
@@ -369,7 +414,7 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
     if (only_bucket && !only_bucket->count(kv.first)) continue;
     const int lay = h->layout[kv.first];
     if (lay < 0) return fail(SIM_EINVAL, "snake too long for the lane layouts (max 128 nodes)");
-    const int G = layout_lanes(lay), per = 32 / G;
+    const int per = lay_wide(h, lay) ? 1 : 32 / layout_lanes(lay);
     for (int s : kv.second) cls[s] = (int)cls_base.size();
     cls_base.push_back((int)order.size());
     for (size_t b = 0; b < kv.second.size(); b += per) {
@@ -392,10 +437,6 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
   });
   std::vector<int4> hitems(its.size());
   for (size_t i = 0; i < its.size(); ++i) hitems[i] = make_int4(its[i].off, its[i].cnt, its[i].lay, 0);
-  for (int4* p : {h->items, h->items0}) if (p) cudaFree(p);
-  for (int* p : {h->order, h->sched_cls, h->sched_base, h->sched_hist, h->sched_key}) if (p) cudaFree(p);
-  h->items = h->items0 = nullptr;
-  h->order = h->sched_cls = h->sched_base = h->sched_hist = h->sched_key = nullptr;
   h->n_items = (int)hitems.size();
   h->n_cls = (int)cls_base.size();
   if (h->n_items > 0) {
@@ -440,25 +481,37 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
   for (const It& it : its) { cnt[it.lay] += 1; work[it.lay] += it.cost * layout_npl(it.lay); }
   h->lay_first[0] = 0;
   for (int l = 0; l < kLayouts; ++l) h->lay_first[l + 1] = h->lay_first[l] + cnt[l];
-  int dev = 0, sms = 0;
-  CU(cudaGetDevice(&dev));
-  CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   h->n_lay = 0;
   for (int l = 0; l < kLayouts; ++l) {
     h->lay_grid[l] = 0;
     if (cnt[l] == 0) continue;
     int per_sm = 0;
     const int var = solver_var(h);
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kSolverKernels[0][var][l], 128,
+    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(h, false, l), 128,
                                                      var == kVarPcr ? pcr_smem_bytes(l) : 0));
     const int need = (cnt[l] + 3) / 4;  // four warps per block
-    h->lay_grid[l] = std::max(1, std::min(need, std::max(1, per_sm) * sms));
+    h->lay_grid[l] = std::max(1, std::min(need, std::max(1, per_sm) * h->sms));
     h->lay_launch[h->n_lay++] = l;
   }
   std::stable_sort(h->lay_launch, h->lay_launch + h->n_lay,
                    [&](int a, int b) { return work[a] > work[b]; });
   h->graph_dirty = true;
   return SIM_OK;
+}
+
+// New layouts or another solver: both sets of items are void.
+SimStatus rebuild_items(SimHandle* h, const std::map<int, int>* only_bucket = nullptr) {
+  h->parked.release();
+  return build_items(h, only_bucket);
+}
+
+// After a change of configuration: the set of items its rule asks for, kept from an earlier
+// use where there is one.
+SimStatus choose_items(SimHandle* h) {
+  if (use_wide(h) == h->wide) return SIM_OK;
+  std::swap(static_cast<ItemSet&>(*h), h->parked);
+  if (h->items && h->wide == use_wide(h)) return SIM_OK;
+  return build_items(h);
 }
 
 SolverArgs make_args(SimHandle* h, int n_steps) {
@@ -495,6 +548,7 @@ SolverArgs make_args(SimHandle* h, int n_steps) {
   A.net_every = std::max(1, h->cfg.net_every);
   A.feat_kinds = feature_kinds(h->cfg.warm, h->cfg.net_rows);
   A.beta_net = h->cfg.beta_net < 0.f ? h->cfg.beta : h->cfg.beta_net;
+  A.order_npl = 1;
   A.span = 1;
   return A;
 }
@@ -597,6 +651,7 @@ SimStatus launch_layout(SimHandle* h, const SolverArgs& A, int l, cudaStream_t s
   B.items = h->items + h->lay_first[l];
   B.n_items = h->lay_first[l + 1] - h->lay_first[l];
   B.work = h->work + l;
+  B.order_npl = layout_npl(l);
   CU(cudaMemsetAsync(B.work, 0, sizeof(int), s));
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   CU(cudaStreamIsCapturing(s, &cap));
@@ -608,7 +663,7 @@ SimStatus launch_layout(SimHandle* h, const SolverArgs& A, int l, cudaStream_t s
     CU(cudaEventRecord(tm.a, s));
   }
   const int var = solver_var(h);
-  kSolverKernels[A.split ? 1 : 0][var][l]<<<h->lay_grid[l], 128, var == kVarPcr ? pcr_smem_bytes(l) : 0, s>>>(B);
+  solver_kernel(h, A.split != 0, l)<<<h->lay_grid[l], 128, var == kVarPcr ? pcr_smem_bytes(l) : 0, s>>>(B);
   CU(cudaGetLastError());
   if (timed) {
     CU(cudaEventRecord(tm.b, s));
@@ -765,6 +820,9 @@ SimStatus sim_create(const SimConfig* cfg, int n_snakes, const SnakeParams* para
     CUC(cudaStreamCreateWithFlags(&h->side[l], cudaStreamNonBlocking));
     CUC(cudaEventCreateWithFlags(&h->ev_side[l], cudaEventDisableTiming));
   }
+  int dev = 0;
+  CUC(cudaGetDevice(&dev));
+  CUC(cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev));
 #undef CUC
   st = build_items(h);
   if (st != SIM_OK) return cleanup(st);
@@ -779,7 +837,7 @@ SimStatus sim_set_config(SimHandle* h, const SimConfig* cfg) {
   const bool regrid = cfg->solver != h->cfg.solver;  // another kernel variant, other occupancy
   h->cfg = *cfg;
   h->graph_dirty = true;
-  return regrid ? build_items(h) : SIM_OK;
+  return regrid ? rebuild_items(h) : choose_items(h);
 }
 
 SimStatus sim_set_pressure(SimHandle* h, const float* u, int is_device) {
@@ -957,7 +1015,7 @@ SimStatus sim_set_layout(SimHandle* h, int nodes, int lanes, int npl) {
   if (!(lanes == 8 || lanes == 16 || lanes == 32) || npl < 1 || npl > 4 || lanes * npl < nodes)
     return fail(SIM_EINVAL, "layout needs lanes in {8,16,32}, nodes_per_lane in 1..4, lanes*npl >= nodes");
   h->layout[nodes] = layout_id(lanes, npl);
-  return build_items(h);
+  return rebuild_items(h);
 }
 
 SimStatus sim_autotune(SimHandle* h, int n_steps) {
@@ -1017,7 +1075,7 @@ SimStatus sim_autotune(SimHandle* h, int n_steps) {
         one[N] = layout_id(G, npl);
         h->layout = layout0;
         h->layout[N] = layout_id(G, npl);
-        if ((st = build_items(h, &one)) != SIM_OK) break;
+        if ((st = rebuild_items(h, &one)) != SIM_OK) break;
         float ms = 0.f;
         for (int rep = 0; rep < 2 && st == SIM_OK; ++rep) {
           if (!xfer(false) || !ok(cudaEventRecord(a, h->stream), "cudaEventRecord")) break;
@@ -1041,7 +1099,7 @@ SimStatus sim_autotune(SimHandle* h, int n_steps) {
   for (void* q : {(void*)p0, (void*)v0, (void*)pr0, (void*)l0, (void*)r0, (void*)i0, (void*)s0})
     if (q) cudaFree(q);
   h->layout = run == SIM_OK ? best : layout0;
-  const SimStatus rebuilt = build_items(h);
+  const SimStatus rebuilt = rebuild_items(h);
   if (run != SIM_OK) return run;
   if (put_back != SIM_OK) return put_back;
   return rebuilt;
@@ -1283,12 +1341,13 @@ SimStatus sim_destroy(SimHandle* h) {
     if (h->ev_side[l]) cudaEventDestroy(h->ev_side[l]);
   }
   void* ptrs[] = {h->pos, h->vel, h->press, h->lam, h->prm, h->node_off_d, h->link_off_d, h->resid,
-                  h->iters, h->status, h->items, h->order, h->ucmd, h->inv_mass_d, h->scratch3,
+                  h->iters, h->status, h->ucmd, h->inv_mass_d, h->scratch3,
                   h->lam0, h->feat, h->snap_pos, h->snap_vel, h->snap_press, h->snap_lam,
-                  h->step_dev, h->snap_step_dev, h->work, h->sched_cls, h->sched_base,
-                  h->sched_hist, h->sched_key, h->items0, h->feat_off_d, h->snap_resid,
+                  h->step_dev, h->snap_step_dev, h->work, h->feat_off_d, h->snap_resid,
                   h->snap_iters, h->snap_status, h->snap_feat, h->train_off};
   for (void* p : ptrs) if (p) cudaFree(p);
+  static_cast<ItemSet*>(h)->release();
+  h->parked.release();
   delete h;
   return SIM_OK;
 }

@@ -168,15 +168,77 @@ __device__ __forceinline__ void friction_limit(const SnakeK& S, float bx, float 
 
 namespace snakesim {
 
+// A layout (G lanes x V nodes per lane) fixes the order in which a node's row contributions are
+// added: a lane adds its own rows' as it walks them, and what the neighbouring lanes' rows
+// give to its first and last node at the end.  The WIDE kernels run such a layout's snakes
+// with more lanes and fewer nodes per lane and add in the same order, so that the result
+// is the same bits: every node knows whether it is the first or last of its V (Roles), the
+// rows' multipliers travel between lanes instead of sums, and gather_wide adds them up.
+template <int NPL>
+struct Roles {
+  bool first[NPL], last[NPL];
+};
+// Gradients of the segments i0 - 1 .. i0 + NPL - 1 of a lane's nodes i0 .. i0 + NPL - 1.
+template <int NPL>
+struct RowGrads {
+  float n[NPL + 1][3], y[NPL + 1][2], p[NPL + 1][3];
+  __device__ __forceinline__ void put(int u, const Seg& s) {
+    n[u][0] = s.nx; n[u][1] = s.ny; n[u][2] = s.nz;
+    y[u][0] = s.gyx; y[u][1] = s.gyy;
+    p[u][0] = s.gpx; p[u][1] = s.gpy; p[u][2] = s.gpz;
+  }
+};
+// acc: the contributions of the rows of node i - 1 (unless i is a first node), i and i + 1
+// (unless i is a last node); endL / endR: those of the rows of i - 1 / i + 1, to be added
+// after the contact and friction rows where i is a first / last node.
+template <int NPL>
+__device__ __forceinline__ void gather_wide(const RowGrads<NPL>& W, const Roles<NPL>& R, const float (&dl)[NPL][6],
+                                            float (&acc)[NPL][3], float (&endL)[NPL][3], float (&endR)[NPL][3]) {
+  float lft[3], rgt[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float v = __shfl_up_sync(kFull, dl[NPL - 1][k], 1);
+    lft[k] = (threadIdx.x & 31) != 0 ? v : 0.f;  // node 0 has no left row
+  }
+#pragma unroll
+  for (int k = 1; k < 3; ++k) {
+    const float v = __shfl_down_sync(kFull, dl[0][k], 1);
+    rgt[k] = (threadIdx.x & 31) != 31 ? v : 0.f;  // nor the warp's last node a right one
+  }
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    const float ls = j > 0 ? dl[j > 0 ? j - 1 : 0][0] : lft[0], ly = j > 0 ? dl[j > 0 ? j - 1 : 0][1] : lft[1],
+                lp = j > 0 ? dl[j > 0 ? j - 1 : 0][2] : lft[2];
+    const float ry = j + 1 < NPL ? dl[j + 1 < NPL ? j + 1 : 0][1] : rgt[1],
+                rp = j + 1 < NPL ? dl[j + 1 < NPL ? j + 1 : 0][2] : rgt[2];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      float c = __fmul_rn(W.n[j][d], ls);
+      if (d < 2) c = fmaf(W.y[j][d], ly, c);
+      c = fmaf(W.p[j][d], lp, c);
+      float a = fmaf(-W.n[j + 1][d], dl[j][0], R.first[j] ? 0.f : c);
+      if (d < 2) a = fmaf(-W.y[j][d] - W.y[j + 1][d], dl[j][1], a);
+      a = fmaf(-W.p[j][d] - W.p[j + 1][d], dl[j][2], a);
+      float b = R.last[j] ? 0.f : a;
+      if (d < 2) b = fmaf(W.y[j + 1][d], ry, b);
+      b = fmaf(W.p[j + 1][d], rp, b);
+      acc[j][d] = R.last[j] ? a : b;
+      endL[j][d] = c;
+      endR[j][d] = b;
+    }
+  }
+}
+
 // Warm-start pass at the predicted positions: uses d_j = lambda_j (zeroing rows that do not
 // exist or touch no free node) and applies it, so that M (x - x~) = J^T lambda.
 // No branches on row existence: every row of every node slot is evaluated (on a straight
 // dummy segment where the segment does not exist) and a row that does not exist contributes
 // d = 0, so that the lane's node slots form independent instruction streams.
-template <int NPL, int G>
+template <int NPL, int G, bool WIDE>
 __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, int q, bool live,
                                           const float (&xs)[NPL][3], float (&dx)[NPL][3], const float (&xsl)[3],
-                                          const float (&xsr)[3], float (&lam)[NPL][6]) {
+                                          const float (&xsr)[3], float (&lam)[NPL][6],
+                                          const Roles<NPL>& R) {
   const float L0 = S.L0;
   // neighbour displacements across the lane boundary
   float dxl[3], dxr[3];
@@ -205,10 +267,13 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
 #pragma unroll
   for (int j = 0; j < NPL; ++j) acc[j][0] = acc[j][1] = acc[j][2] = 0.f;
   Seg sp = seg(0);  // segment i0 - 1
+  RowGrads<NPL> W;
+  if (WIDE) W.put(0, sp);
 #pragma unroll
   for (int j = 0; j < NPL; ++j) {
     const int i = i0 + j;
     const Seg sc = seg(j + 1);  // segment i
+    if (WIDE) W.put(j + 1, sc);
     const bool act = live && i < S.N;
     const float wi = (i < S.nfix) ? 0.f : S.inv_m;
     const float wl = (i - 1 < S.nfix) ? 0.f : S.inv_m;
@@ -218,8 +283,10 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
     {
       const float d = act && i + 1 <= S.N - 1 && wi + wr > 0.f ? lam[j][0] : 0.f;
       lam[j][0] = d;
-      acc[j][0] -= sc.nx * d; acc[j][1] -= sc.ny * d; acc[j][2] -= sc.nz * d;
-      tr[0] += sc.nx * d; tr[1] += sc.ny * d; tr[2] += sc.nz * d;
+      if (!WIDE) {
+        acc[j][0] -= sc.nx * d; acc[j][1] -= sc.ny * d; acc[j][2] -= sc.nz * d;
+        tr[0] += sc.nx * d; tr[1] += sc.ny * d; tr[2] += sc.nz * d;
+      }
     }
     const bool bend = act && i >= 1 && i <= S.N - 2;
     {
@@ -230,9 +297,11 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
                        wr * (g2x * g2x + g2y * g2y);
       const float d = bend && wg > 0.f ? lam[j][1] : 0.f;
       lam[j][1] = d;
-      tl[0] += g0x * d; tl[1] += g0y * d;
-      acc[j][0] += g1x * d; acc[j][1] += g1y * d;
-      tr[0] += g2x * d; tr[1] += g2y * d;
+      if (!WIDE) {
+        tl[0] += g0x * d; tl[1] += g0y * d;
+        acc[j][0] += g1x * d; acc[j][1] += g1y * d;
+        tr[0] += g2x * d; tr[1] += g2y * d;
+      }
     }
     {
       const float g0x = sp.gpx, g0y = sp.gpy, g0z = sp.gpz;
@@ -243,12 +312,16 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
                        wr * (g2x * g2x + g2y * g2y + g2z * g2z);
       const float d = bend && wg > 0.f ? lam[j][2] : 0.f;
       lam[j][2] = d;
-      tl[0] += g0x * d; tl[1] += g0y * d; tl[2] += g0z * d;
-      acc[j][0] += g1x * d; acc[j][1] += g1y * d; acc[j][2] += g1z * d;
-      tr[0] += g2x * d; tr[1] += g2y * d; tr[2] += g2z * d;
+      if (!WIDE) {
+        tl[0] += g0x * d; tl[1] += g0y * d; tl[2] += g0z * d;
+        acc[j][0] += g1x * d; acc[j][1] += g1y * d; acc[j][2] += g1z * d;
+        tr[0] += g2x * d; tr[1] += g2y * d; tr[2] += g2z * d;
+      }
     }
     sp = sc;
   }
+  float endL[NPL][3], endR[NPL][3];
+  if (WIDE) gather_wide<NPL>(W, R, lam, acc, endL, endR);
 #pragma unroll
   for (int j = 0; j < NPL; ++j) {
     const int i = i0 + j;
@@ -263,15 +336,20 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
   float fromR[3], fromL[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    fromR[d] = __shfl_down_sync(kFull, accL[d], 1, G);  // right lane's rows -> my last node
-    fromL[d] = __shfl_up_sync(kFull, accR[d], 1, G);    // left lane's rows -> my first node
+    fromR[d] = WIDE ? 0.f : __shfl_down_sync(kFull, accL[d], 1, G);  // right lane's rows -> my last node
+    fromL[d] = WIDE ? 0.f : __shfl_up_sync(kFull, accR[d], 1, G);    // left lane's rows -> my first node
   }
 #pragma unroll
   for (int j = 0; j < NPL; ++j) {
     const int i = i0 + j;
     float ax = acc[j][0], ay = acc[j][1], az = acc[j][2];
-    if (j == 0 && q > 0) { ax += fromL[0]; ay += fromL[1]; az += fromL[2]; }
-    if (j == NPL - 1 && q < G - 1) { ax += fromR[0]; ay += fromR[1]; az += fromR[2]; }
+    if (WIDE) {
+      if (R.first[j]) { ax += endL[j][0]; ay += endL[j][1]; az += endL[j][2]; }
+      if (R.last[j]) { ax += endR[j][0]; ay += endR[j][1]; az += endR[j][2]; }
+    } else {
+      if (j == 0 && q > 0) { ax += fromL[0]; ay += fromL[1]; az += fromL[2]; }
+      if (j == NPL - 1 && q < G - 1) { ax += fromR[0]; ay += fromR[1]; az += fromR[2]; }
+    }
     const bool on = live && i < S.N;
     const float wi = (i < S.nfix) ? 0.f : S.inv_m;
     dx[j][0] = on ? dx[j][0] + wi * ax : dx[j][0];
@@ -300,11 +378,11 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
 // form, same bits: one 41-node snake at ten updates 256 -> 200 us per env-step, 4096 uneven
 // snakes 785 -> 600 us; 8192 snakes to 1e-4 cold 49-58 -> 32-35 ms, 256 cantilevers to 1e-6
 // 30.9 -> 18.8 ms.
-template <int NPL, int G, bool ANISO>
+template <int NPL, int G, bool ANISO, bool WIDE>
 __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int q, bool valid,
                                        const float (&xs)[NPL][3], float (&dx)[NPL][3], const float (&xsl)[3],
                                        const float (&xsr)[3], float (&lam)[NPL][6], const float (&th)[NPL],
-                                       float& r_end, int& updates) {
+                                       const Roles<NPL>& R, float& r_end, int& updates) {
   const float L0 = S.L0;
   const int i0 = q * NPL;
   const unsigned lane = threadIdx.x & 31u;
@@ -380,21 +458,27 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     for (int j = 0; j < NPL; ++j) acc[j][0] = acc[j][1] = acc[j][2] = 0.f;
     float r = 0.f;
     Seg sp = seg(0);  // segment i0 - 1
+    RowGrads<NPL> W;
+    float endL[NPL][3], endR[NPL][3];
+    if (WIDE) W.put(0, sp);
 #pragma unroll
     for (int j = 0; j < NPL; ++j) {
       const Seg sc = seg(j + 1);  // segment i
+      if (WIDE) W.put(j + 1, sc);
       const float wl = w[j], wi = w[j + 1], wr = w[j + 2];
       float* tl = (j > 0) ? acc[j - 1] : accL;        // node i-1
       float* tr = (j + 1 < NPL) ? acc[j + 1] : accR;  // node i+1
       // ---- stretch (i, i+1): c = |e| - L0 (Eq. 3 with a constant rest length)
       {
-        const float c = sc.len - L0;
+        const float c = __fsub_rn(sc.len, L0);
         const float l = lam[j][0];
         r = fmaxf(r, fabsf(c + S.at_s * l) * ws[j]);
         const float d = __fmul_rn(A.omega * (-c - S.at_s * l), rs[j]);
         dl[j][0] = d;
-        acc[j][0] -= sc.nx * d; acc[j][1] -= sc.ny * d; acc[j][2] -= sc.nz * d;
-        tr[0] += sc.nx * d; tr[1] += sc.ny * d; tr[2] += sc.nz * d;
+        if (!WIDE) {
+          acc[j][0] -= sc.nx * d; acc[j][1] -= sc.ny * d; acc[j][2] -= sc.nz * d;
+          tr[0] += sc.nx * d; tr[1] += sc.ny * d; tr[2] += sc.nz * d;
+        }
       }
       // ---- yaw and pitch bend centred on node i (rows in length units: L0 x angle)
       // yaw: L0 (atan2(z . (e1 x e2), e1_h . e2_h) - theta_rest)
@@ -411,9 +495,11 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
         r = fmaxf(r, fabsf(c + S.at_b * l) * wb[j]);
         const float d = __fmul_rn(A.omega * (-c - S.at_b * l), rcp_approx(wg + ab[j]));
         dl[j][1] = d;
-        tl[0] += g0x * d; tl[1] += g0y * d;
-        acc[j][0] += g1x * d; acc[j][1] += g1y * d;
-        tr[0] += g2x * d; tr[1] += g2y * d;
+        if (!WIDE) {
+          tl[0] += g0x * d; tl[1] += g0y * d;
+          acc[j][0] += g1x * d; acc[j][1] += g1y * d;
+          tr[0] += g2x * d; tr[1] += g2y * d;
+        }
       }
       // pitch: L0 (elevation(e2) - elevation(e1))
       {
@@ -428,12 +514,15 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
         r = fmaxf(r, fabsf(c + S.at_b * l) * wb[j]);
         const float d = __fmul_rn(A.omega * (-c - S.at_b * l), rcp_approx(wg + ab[j]));
         dl[j][2] = d;
-        tl[0] += g0x * d; tl[1] += g0y * d; tl[2] += g0z * d;
-        acc[j][0] += g1x * d; acc[j][1] += g1y * d; acc[j][2] += g1z * d;
-        tr[0] += g2x * d; tr[1] += g2y * d; tr[2] += g2z * d;
+        if (!WIDE) {
+          tl[0] += g0x * d; tl[1] += g0y * d; tl[2] += g0z * d;
+          acc[j][0] += g1x * d; acc[j][1] += g1y * d; acc[j][2] += g1z * d;
+          tr[0] += g2x * d; tr[1] += g2y * d; tr[2] += g2z * d;
+        }
       }
       sp = sc;
     }
+    if (WIDE) gather_wide<NPL>(W, R, dl, acc, endL, endR);
     // a group could stop only if none of its lanes has a bilateral term over the tolerance
     // (a non-finite term counts as not over, so that it reaches the residual)
     const unsigned over_b = __ballot_sync(kFull, r * S.inv_L0 > A.tol);
@@ -503,14 +592,19 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
       float fromR[3], fromL[3];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        fromR[d] = __shfl_down_sync(kFull, accL[d], 1, G);  // right lane's rows -> my last node
-        fromL[d] = __shfl_up_sync(kFull, accR[d], 1, G);    // left lane's rows -> my first node
+        fromR[d] = WIDE ? 0.f : __shfl_down_sync(kFull, accL[d], 1, G);  // right lane's rows -> my last node
+        fromL[d] = WIDE ? 0.f : __shfl_up_sync(kFull, accR[d], 1, G);    // left lane's rows -> my first node
       }
 #pragma unroll
       for (int j = 0; j < NPL; ++j) {
         float ax = acc[j][0], ay = acc[j][1], az = acc[j][2];
-        if (j == 0 && q > 0) { ax += fromL[0]; ay += fromL[1]; az += fromL[2]; }
-        if (j == NPL - 1 && q < G - 1) { ax += fromR[0]; ay += fromR[1]; az += fromR[2]; }
+        if (WIDE) {
+          if (R.first[j]) { ax += endL[j][0]; ay += endL[j][1]; az += endL[j][2]; }
+          if (R.last[j]) { ax += endR[j][0]; ay += endR[j][1]; az += endR[j][2]; }
+        } else {
+          if (j == 0 && q > 0) { ax += fromL[0]; ay += fromL[1]; az += fromL[2]; }
+          if (j == NPL - 1 && q < G - 1) { ax += fromR[0]; ay += fromR[1]; az += fromR[2]; }
+        }
         const float wi = w[j + 1];
         if (G == 32 || live) {  // a group that has stopped keeps its state
           dx[j][0] = dx[j][0] + wi * ax;
@@ -812,7 +906,7 @@ __device__ void newton_pcr(const SnakeK& S, const SolverArgs& A, int q, bool val
 // preconditioned conjugate residual over the bilateral rows (contact-free substeps;
 // `smem` is its per-block shared-memory area).
 enum { kVarJacobi = 0, kVarAniso = 1, kVarPcr = 2 };
-template <int NPL, int G, bool SPLIT, int VAR>
+template <int NPL, int G, bool SPLIT, int VAR, bool WIDE>
 __device__ void run_group(const SolverArgs& A, int snake, bool valid, float* smem) {
   constexpr bool ANISO = VAR == kVarAniso;
   const int lane = threadIdx.x & 31;
@@ -837,6 +931,14 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid, float* sme
   S.e_inf = expf(-h / P.tau_inf); S.e_def = expf(-h / P.tau_def);
   S.om_m = A.omega * S.mass;
   S.damp_over_h = expf(-P.damping * h) / h;
+
+  Roles<NPL> R;  // WIDE: this lane's nodes in the layout whose order of sums is kept
+#pragma unroll
+  for (int j = 0; j < NPL; ++j) {
+    const int m = WIDE ? (q * NPL + j) % A.order_npl : 0;
+    R.first[j] = WIDE && m == 0;
+    R.last[j] = WIDE && m == A.order_npl - 1;
+  }
 
   // x = xs + dx; between substeps dx holds the last substep's displacement
   float xs[NPL][3], dx[NPL][3], v[NPL][3], lam[NPL][6], pR[NPL], pL[NPL], th[NPL];
@@ -892,7 +994,11 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid, float* sme
           u = A.ucmd[S.lb + kl];
         } else {
           // argument reduced to [-pi, pi] first, where the fast sine is accurate to ~1e-6
-          float arg = phase + (float)kl * P.gait_lag;
+          // (rounded as in the layout's own kernel: with one node per lane the phase's product
+          // is the fused one)
+          float arg = !WIDE ? phase + (float)kl * P.gait_lag
+                            : (A.order_npl > 1 ? fmaf((float)kl, P.gait_lag, phase)
+                                               : fmaf(6.283185307179586f, (float)cyc, (float)kl * P.gait_lag));
           arg -= 6.283185307179586f * rintf(arg * 0.15915494309189535f);
           float a = P.gait_offset + P.gait_scale * __sinf(arg);
           a = fminf(1.f, fmaxf(-1.f, a)) * P.gait_amp;
@@ -952,14 +1058,14 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid, float* sme
           lam[j][k] = l;
         }
       }
-      warm_pass<NPL, G>(S, A, q, valid, xs, dx, xsl, xsr, lam);
+      warm_pass<NPL, G, WIDE>(S, A, q, valid, xs, dx, xsl, xsr, lam, R);
     }
     float rs = 0.f;
     int ks = 0;
     if (VAR == kVarPcr) {
       newton_pcr<NPL, G>(S, A, q, valid, xs, dx, lam, th, smem, rs, ks);
     } else {
-      jacobi<NPL, G, ANISO>(S, A, q, valid, xs, dx, xsl, xsr, lam, th, rs, ks);
+      jacobi<NPL, G, ANISO, WIDE>(S, A, q, valid, xs, dx, xsl, xsr, lam, th, R, rs, ks);
     }
     // a non-finite displacement anywhere in the snake marks the step (fmaxf drops NaN)
     float bad = 0.f;

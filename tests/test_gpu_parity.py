@@ -521,3 +521,35 @@ def test_benchmark_configuration_sampled_parity():
         assert (np.abs(sub.st["iters"] - o.iters) <= np.maximum(0.05 * o.iters, 20)).all(), (cfg, sub.st["iters"], o.iters)
     g.close()
     net.close()
+
+
+@pytest.mark.parametrize("lanes,npl", [(8, 1), (8, 2), (8, 3), (8, 4), (16, 1), (16, 2), (16, 3), (16, 4)])
+@pytest.mark.parametrize("mode", ["cold", "previous", "aniso"])
+def test_one_snake_per_warp_gives_the_layouts_bits(lanes, npl, mode):
+    """The snakes of an 8- or 16-lane layout run one per warp in small batches (and to a
+    tolerance) and several per warp in large ones at fixed updates: the same bits either way,
+    for the shortest and longest snakes of the layout and some between, and through a
+    change of the tolerance that switches between the two on one handle."""
+    longest = lanes * npl
+    n = np.unique(np.linspace(2, longest, 7).astype(int))
+    small = W.batched(n=len(n), seed=50, links=(1, 1))
+    small["seg_per_link"][:] = n - 1
+    if mode == "aniso":
+        small["mu_side"] = np.where(np.arange(len(n)) % 2 == 0, 3.0 * small["mu"], 0.0)
+    copies = 16 * torch.cuda.get_device_properties(0).multi_processor_count // len(n) + 1
+    big = {k: np.tile(v, copies) for k, v in small.items()}
+    s = W.solver_settings(iters=10, warm=1 if mode == "previous" else 0, beta=0.75)
+    a, b = Sim(small, s), Sim(big, s)
+    for g in (a, b):
+        for N in n:
+            g.set_layout(int(N), lanes, npl)
+        g.step(2)
+        g.set_config(iters=40, tol=1e-3)
+        g.step(1)
+        g.set_config(iters=10, tol=0.0)
+        g.step(1, graph=True)
+    sa, sb = a.state_host(), b.state_host()
+    for k in ("pos", "vel", "resid", "iters"):
+        assert np.array_equal(sa[k], sb[k][:len(sa[k])]), k
+        assert np.array_equal(sa[k], sb[k][-len(sa[k]):]), k
+    assert torch.equal(a.lam(), b.lam()[:a.n_nodes])
