@@ -70,7 +70,6 @@ namespace {
 // order of sums (see Roles in solver.cuh).
 template <int NPL, int G, bool SPLIT, int VAR, bool WIDE = false>
 __global__ void __launch_bounds__(128, SNAKE_MIN_BLOCKS) snake_solver_kernel(SolverArgs A) {
-  extern __shared__ float solver_smem[];  // Newton + PCR only (kPcrFloatsPerSlot x 32 NPL per warp)
   const int lane = threadIdx.x & 31;
   for (;;) {
     int it = 0;
@@ -81,7 +80,7 @@ __global__ void __launch_bounds__(128, SNAKE_MIN_BLOCKS) snake_solver_kernel(Sol
     const int gi = lane / G;
     const bool ok = gi < item.y;
     const int snake = ok ? A.order[item.x + gi] : 0;
-    run_group<NPL, G, SPLIT, VAR, WIDE>(A, snake, ok, solver_smem);
+    run_group<NPL, G, SPLIT, VAR, WIDE>(A, snake, ok);
   }
 }
 
@@ -103,8 +102,6 @@ const SolverKernel kWideKernels[2][2][2] = {
      {snake_solver_kernel<1, 32, false, kVarAniso, true>, snake_solver_kernel<2, 32, false, kVarAniso, true>}},
     {{snake_solver_kernel<1, 32, true, kVarJacobi, true>, snake_solver_kernel<2, 32, true, kVarJacobi, true>},
      {snake_solver_kernel<1, 32, true, kVarAniso, true>, snake_solver_kernel<2, 32, true, kVarAniso, true>}}};
-// dynamic shared memory of a block of the Newton + PCR kernels
-inline size_t pcr_smem_bytes(int lay) { return (size_t)4 * kPcrFloatsPerSlot * 32 * layout_npl(lay) * sizeof(float); }
 #undef SNAKE_KERNELS
 
 // ------------------------------------------------------------------ scheduling
@@ -486,9 +483,7 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
     h->lay_grid[l] = 0;
     if (cnt[l] == 0) continue;
     int per_sm = 0;
-    const int var = solver_var(h);
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(h, false, l), 128,
-                                                     var == kVarPcr ? pcr_smem_bytes(l) : 0));
+    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(h, false, l), 128, 0));
     const int need = (cnt[l] + 3) / 4;  // four warps per block
     h->lay_grid[l] = std::max(1, std::min(need, std::max(1, per_sm) * h->sms));
     h->lay_launch[h->n_lay++] = l;
@@ -662,8 +657,7 @@ SimStatus launch_layout(SimHandle* h, const SolverArgs& A, int l, cudaStream_t s
     CU(cudaEventCreate(&tm.b));
     CU(cudaEventRecord(tm.a, s));
   }
-  const int var = solver_var(h);
-  solver_kernel(h, A.split != 0, l)<<<h->lay_grid[l], 128, var == kVarPcr ? pcr_smem_bytes(l) : 0, s>>>(B);
+  solver_kernel(h, A.split != 0, l)<<<h->lay_grid[l], 128, 0, s>>>(B);
   CU(cudaGetLastError());
   if (timed) {
     CU(cudaEventRecord(tm.b, s));

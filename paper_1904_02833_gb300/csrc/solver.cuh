@@ -740,54 +740,58 @@ __device__ __forceinline__ float chamber_law(float p, float t, const SolverArgs&
   return p;
 }
 
+__device__ __forceinline__ void pcr_put(PcrSeg& o, bool on, const Seg& s) {
+  const float g[8] = {s.nx, s.ny, s.nz, s.gyx, s.gyy, s.gpx, s.gpy, s.gpz};
+#pragma unroll
+  for (int c = 0; c < 8; ++c) o.g[c] = on ? g[c] : 0.f;
+}
+
 // Newton + PCR solve of one contact-free substep (see pcr.cuh) for the snake of this lane
 // group, from the current multipliers and displacements; returns the final normalised
 // residual and the number of matrix-vector products.
 template <int NPL, int G>
 __device__ void newton_pcr(const SnakeK& S, const SolverArgs& A, int q, bool valid,
                            const float (&xs)[NPL][3], float (&dx)[NPL][3], float (&lam)[NPL][6],
-                           const float (&th)[NPL], float* smem, float& r_end, int& mv) {
-  const int lane = threadIdx.x & 31;
-  const PcrSmem M = pcr_smem(smem, NPL);
-  const int base = (lane / G) * G * NPL;
+                           const float (&th)[NPL], float& r_end, int& mv) {
   const float L0 = S.L0;
   float x[NPL][3], z[NPL][3], p[NPL][3], qv[NPL][3], iD[NPL][3], y[NPL][3], u[NPL][3];
+  PcrSeg sg[NPL + 1];
   bool gdone = !valid;
   mv = 0;
   r_end = 0.f;
   for (;;) {
     // ---- linearise at x = x_s + d: segments, rows, preconditioner, right-hand side
+    float xl[3], dxl[3], xr[3], dxr[3];  // nodes before and after the lane's
 #pragma unroll
-    for (int j = 0; j < NPL; ++j)
-#pragma unroll
-      for (int d = 0; d < 3; ++d) { M.U(d, base + q * NPL + j) = xs[j][d]; M.U(3 + d, base + q * NPL + j) = dx[j][d]; }
-    __syncwarp();
+    for (int d = 0; d < 3; ++d) {
+      xl[d] = __shfl_up_sync(kFull, xs[NPL - 1][d], 1, G);
+      dxl[d] = __shfl_up_sync(kFull, dx[NPL - 1][d], 1, G);
+      xr[d] = __shfl_down_sync(kFull, xs[0][d], 1, G);
+      dxr[d] = __shfl_down_sync(kFull, dx[0][d], 1, G);
+    }
     float r = 0.f;
     Seg sp = make_seg(1.f, 0.f, 0.f, L0);
-    {
-      const int i0 = q * NPL, s0 = base + i0;
-      if (valid && i0 >= 1 && i0 <= S.N - 1)
-        sp = make_seg((M.U(0, s0) - M.U(0, s0 - 1)) + (M.U(3, s0) - M.U(3, s0 - 1)),
-                      (M.U(1, s0) - M.U(1, s0 - 1)) + (M.U(4, s0) - M.U(4, s0 - 1)),
-                      (M.U(2, s0) - M.U(2, s0 - 1)) + (M.U(5, s0) - M.U(5, s0 - 1)), L0);
-    }
+    const bool has_left = valid && q * NPL >= 1 && q * NPL <= S.N - 1;
+    if (has_left)
+      sp = make_seg((xs[0][0] - xl[0]) + (dx[0][0] - dxl[0]), (xs[0][1] - xl[1]) + (dx[0][1] - dxl[1]),
+                    (xs[0][2] - xl[2]) + (dx[0][2] - dxl[2]), L0);
+    pcr_put(sg[0], has_left, sp);
 #pragma unroll
     for (int j = 0; j < NPL; ++j) {
-      const int i = q * NPL + j, s = base + i;
+      const int i = q * NPL + j;
       const bool act = valid && i < S.N;
       const float wi = (i < S.nfix) ? 0.f : S.inv_m;
       const float wl = (i - 1 < S.nfix) ? 0.f : S.inv_m;
       const float wr = (i + 1 < S.nfix) ? 0.f : S.inv_m;
       const bool has_seg = act && i + 1 <= S.N - 1;
       Seg sc = make_seg(1.f, 0.f, 0.f, L0);
+      const float* xn = j + 1 < NPL ? xs[j + 1 < NPL ? j + 1 : 0] : xr;
+      const float* dn = j + 1 < NPL ? dx[j + 1 < NPL ? j + 1 : 0] : dxr;
       if (has_seg)
-        sc = make_seg((M.U(0, s + 1) - xs[j][0]) + (M.U(3, s + 1) - dx[j][0]),
-                      (M.U(1, s + 1) - xs[j][1]) + (M.U(4, s + 1) - dx[j][1]),
-                      (M.U(2, s + 1) - xs[j][2]) + (M.U(5, s + 1) - dx[j][2]), L0);
+        sc = make_seg((xn[0] - xs[j][0]) + (dn[0] - dx[j][0]), (xn[1] - xs[j][1]) + (dn[1] - dx[j][1]),
+                      (xn[2] - xs[j][2]) + (dn[2] - dx[j][2]), L0);
       // segment i's gradients for the products (zero where there is no segment)
-      M.S(0, s) = has_seg ? sc.nx : 0.f; M.S(1, s) = has_seg ? sc.ny : 0.f; M.S(2, s) = has_seg ? sc.nz : 0.f;
-      M.S(3, s) = has_seg ? sc.gyx : 0.f; M.S(4, s) = has_seg ? sc.gyy : 0.f;
-      M.S(5, s) = has_seg ? sc.gpx : 0.f; M.S(6, s) = has_seg ? sc.gpy : 0.f; M.S(7, s) = has_seg ? sc.gpz : 0.f;
+      pcr_put(sg[j + 1], has_seg, sc);
       float b[3] = {0.f, 0.f, 0.f};
       iD[j][0] = iD[j][1] = iD[j][2] = 0.f;
       if (has_seg && wi + wr > 0.f) {  // stretch
@@ -828,11 +832,10 @@ __device__ void newton_pcr(const SnakeK& S, const SolverArgs& A, int q, bool val
     }
     if (!(r <= 3.0e38f)) r = INFINITY;
     r = group_max<G>(r);
-    __syncwarp();
     if (!gdone && (r <= A.tol || mv >= A.K)) { gdone = true; r_end = r; }
     if (__all_sync(kFull, gdone)) break;
     // ---- PCR on (J M^-1 J^T + alpha~) dlambda = b, diagonal preconditioner, from 0
-    pcr_matvec<NPL>(S, M, q, base, valid, iD, z, y, u);
+    pcr_matvec<NPL, G>(S, sg, q, valid, iD, z, y);
     if (!gdone) ++mv;
     float zaz = 0.f;
 #pragma unroll
@@ -856,7 +859,7 @@ __device__ void newton_pcr(const SnakeK& S, const SolverArgs& A, int q, bool val
       for (int j = 0; j < NPL; ++j)
 #pragma unroll
         for (int k = 0; k < 3; ++k) { x[j][k] += alpha * p[j][k]; z[j][k] -= alpha * qv[j][k] * iD[j][k]; }
-      pcr_matvec<NPL>(S, M, q, base, valid, iD, z, y, u);
+      pcr_matvec<NPL, G>(S, sg, q, valid, iD, z, y);
       if (go) ++mv;
       float zaz2 = 0.f;
 #pragma unroll
@@ -876,13 +879,7 @@ __device__ void newton_pcr(const SnakeK& S, const SolverArgs& A, int q, bool val
         }
     }
     // ---- lambda += dlambda, d += M^-1 J^T dlambda (gradients at the linearisation point)
-#pragma unroll
-    for (int j = 0; j < NPL; ++j)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) M.V(k, base + q * NPL + j) = x[j][k];
-    __syncwarp();
-    pcr_jt<NPL>(S, M, q, base, valid, u);
-    __syncwarp();
+    pcr_jt<NPL, G>(S, sg, q, valid, x, u);
     if (!gdone) {
 #pragma unroll
       for (int j = 0; j < NPL; ++j) {
@@ -903,11 +900,10 @@ __device__ void newton_pcr(const SnakeK& S, const SolverArgs& A, int q, bool val
 // VAR: which solve the kernel carries.  kVarJacobi: the Jacobi relaxation with isotropic
 // friction; kVarAniso: the same with the anisotropic friction path (batches where some
 // snake has mu_side > 0; the other kernels carry none of its code); kVarPcr: Newton +
-// preconditioned conjugate residual over the bilateral rows (contact-free substeps;
-// `smem` is its per-block shared-memory area).
+// preconditioned conjugate residual over the bilateral rows (contact-free substeps).
 enum { kVarJacobi = 0, kVarAniso = 1, kVarPcr = 2 };
 template <int NPL, int G, bool SPLIT, int VAR, bool WIDE>
-__device__ void run_group(const SolverArgs& A, int snake, bool valid, float* smem) {
+__device__ void run_group(const SolverArgs& A, int snake, bool valid) {
   constexpr bool ANISO = VAR == kVarAniso;
   const int lane = threadIdx.x & 31;
   const int q = lane & (G - 1);
@@ -1063,7 +1059,7 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid, float* sme
     float rs = 0.f;
     int ks = 0;
     if (VAR == kVarPcr) {
-      newton_pcr<NPL, G>(S, A, q, valid, xs, dx, lam, th, smem, rs, ks);
+      newton_pcr<NPL, G>(S, A, q, valid, xs, dx, lam, th, rs, ks);
     } else {
       jacobi<NPL, G, ANISO, WIDE>(S, A, q, valid, xs, dx, xsl, xsr, lam, th, R, rs, ks);
     }
