@@ -57,7 +57,8 @@ struct SolverArgs {
   const int* order;       // snake indices grouped by layout
   const int* feat_off;    // [snakes] first node of the snake in the feature / lam0 row order
   int n_items;
-  int* work;              // work-queue counter of this launch (zeroed before the launch)
+  int* work;              // work-queue counter of this launch (zeroed before the launch), or
+                          // null: warp w of the grid takes item w
   const float* ucmd;      // [links] command override or null
   const float* lam0;      // learned warm start, normalised multipliers [nodes][6] or null
   __nv_bfloat16* feat;    // warm-start features [nodes * 6][32] (split mode)

@@ -65,16 +65,19 @@ namespace {
 #define SNAKE_MIN_BLOCKS 2
 #endif
 // Persistent: every warp takes the next work item (32/G snakes of one node count) from
-// the layout's counter in global memory until none is left.
+// the layout's counter in global memory until none is left.  Without a counter (a batch
+// whose items all have a warp at once) every warp takes the item of its own number.
 // WIDE (G = 32): the snakes of a layout with fewer lanes, one per warp, in that layout's
 // order of sums (see Roles in solver.cuh).
 template <int NPL, int G, bool SPLIT, int VAR, bool WIDE = false>
 __global__ void __launch_bounds__(128, SNAKE_MIN_BLOCKS) snake_solver_kernel(SolverArgs A) {
   const int lane = threadIdx.x & 31;
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(A.work, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
+  for (int turn = 0;; ++turn) {
+    int it = turn == 0 ? (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) : A.n_items;
+    if (A.work) {
+      if (lane == 0) it = atomicAdd(A.work, 1);
+      it = __shfl_sync(0xffffffffu, it, 0);
+    }
     if (it >= A.n_items) break;
     const int4 item = A.items[it];
     const int gi = lane / G;
@@ -257,6 +260,11 @@ struct ItemSet {
   int lay_launch[kLayouts] = {};      // layouts with work, most work first
   int n_lay = 0;
   bool wide = false;                  // the 8- and 16-lane layouts run by WIDE kernels
+  // Every item is one snake and all of them are resident at once, in blocks of one warp: then
+  // neither grouping nor order matters, and a step needs no work queue (one snake, a captured
+  // env-step: 140 us with the queue's kernel and the counter's clear before the solver,
+  // 130 us without).
+  bool direct = false;
   void release() {
     for (void* p : {(void*)items, (void*)items0, (void*)order, (void*)sched_cls, (void*)sched_base,
                     (void*)sched_hist, (void*)sched_key})
@@ -479,13 +487,16 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
   h->lay_first[0] = 0;
   for (int l = 0; l < kLayouts; ++l) h->lay_first[l + 1] = h->lay_first[l] + cnt[l];
   h->n_lay = 0;
+  h->direct = its.size() <= (size_t)8 * h->sms;  // the warps that two blocks per SM leave room for
+  for (int l = 0; l < kLayouts; ++l)
+    if (cnt[l] > 0 && layout_lanes(l) < 32 && !lay_wide(h, l)) h->direct = false;
   for (int l = 0; l < kLayouts; ++l) {
     h->lay_grid[l] = 0;
     if (cnt[l] == 0) continue;
     int per_sm = 0;
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(h, false, l), 128, 0));
-    const int need = (cnt[l] + 3) / 4;  // four warps per block
-    h->lay_grid[l] = std::max(1, std::min(need, std::max(1, per_sm) * h->sms));
+    const int need = h->direct ? cnt[l] : (cnt[l] + 3) / 4;  // four warps per block
+    h->lay_grid[l] = h->direct ? need : std::max(1, std::min(need, std::max(1, per_sm) * h->sms));
     h->lay_launch[h->n_lay++] = l;
   }
   std::stable_sort(h->lay_launch, h->lay_launch + h->n_lay,
@@ -576,7 +587,7 @@ SimStatus launch_split(SimHandle* h, int sub, cudaStream_t st, bool net) {
 
 // Rebuilds the work queue from the last env-step's update counts.
 SimStatus schedule(SimHandle* h, cudaStream_t st) {
-  if (h->n_items == 0) return SIM_OK;
+  if (h->n_items == 0 || h->direct) return SIM_OK;
   SchedArgs a;
   a.iters = h->iters; a.node_off = h->node_off_d; a.cls = h->sched_cls; a.cls_base = h->sched_base;
   a.items0 = h->items0; a.hist = h->sched_hist; a.key = h->sched_key; a.order = h->order;
@@ -645,9 +656,9 @@ SimStatus launch_layout(SimHandle* h, const SolverArgs& A, int l, cudaStream_t s
   SolverArgs B = A;
   B.items = h->items + h->lay_first[l];
   B.n_items = h->lay_first[l + 1] - h->lay_first[l];
-  B.work = h->work + l;
+  B.work = h->direct ? nullptr : h->work + l;
   B.order_npl = layout_npl(l);
-  CU(cudaMemsetAsync(B.work, 0, sizeof(int), s));
+  if (B.work) CU(cudaMemsetAsync(B.work, 0, sizeof(int), s));
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   CU(cudaStreamIsCapturing(s, &cap));
   const bool timed = h->timing && cap == cudaStreamCaptureStatusNone;
@@ -657,7 +668,7 @@ SimStatus launch_layout(SimHandle* h, const SolverArgs& A, int l, cudaStream_t s
     CU(cudaEventCreate(&tm.b));
     CU(cudaEventRecord(tm.a, s));
   }
-  solver_kernel(h, A.split != 0, l)<<<h->lay_grid[l], 128, 0, s>>>(B);
+  solver_kernel(h, A.split != 0, l)<<<h->lay_grid[l], h->direct ? 32 : 128, 0, s>>>(B);
   CU(cudaGetLastError());
   if (timed) {
     CU(cudaEventRecord(tm.b, s));
