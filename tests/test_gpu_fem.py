@@ -69,6 +69,14 @@ def test_small_mesh_more_substeps_and_iterations():
     _check(M, w, s, frames=2)
 
 
+def test_chamber_pressures_of_many_substeps():
+    """37 substeps: the pressures are evaluated for 16 substeps at a time."""
+    M = W.fem_link_mesh(m=4, n_sec=3, length=0.03)
+    w = W.fem_links(3, seed=18)
+    w["press_freq"][:] = [7.0, 0.3, 20.0]
+    _check(M, w, W.fem_settings(n_sub=37, iters=12, pcr_iters=12), frames=2)
+
+
 def test_compliant_rows_and_clamped_command():
     """Compliant centre-layer and perimeter rows, offsets that saturate the command
     (clamp at +-1) and a link whose command is exactly zero, over three frames."""
