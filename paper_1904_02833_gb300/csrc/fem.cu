@@ -4,14 +4,16 @@
 // Layout of a block: thread `tid` owns the elements tid + s * blockDim (s < kTPT) and
 // keeps their polar rotations and PCR vectors (z, p, q, A z and the Newton increment,
 // six rows each) in registers.  Shared memory holds the mesh (shape-function gradients,
-// volumes, vertex ids, distance rows, the particle -> contribution-slot lists), the
+// volumes, vertex ids, distance rows), the
 // particles (positions, substep-start positions, velocities, inverse masses, M^-1 J^T v),
 // the elements' multipliers and inverse diagonals, and all vectors of the distance rows.
 //
 // A product y = (J M^-1 J^T + E / h^2) v runs in three phases separated by barriers:
 //  A. every row writes its gradient times v into its contribution slots (element e,
 //     vertex a: R Sigma(v_e) g_a; distance row d: -n v_d, +n v_d);
-//  B. every particle sums its slots in a fixed order and scales by its inverse mass;
+//  B. every particle sums its slots in a fixed order and scales by its inverse mass (the
+//     slot lists are read from global memory: every block reads the same ones, and they
+//     stay in L1);
 //  C. every row reads the sums at its particles: element rows Voigt(sym(R^T H)) with
 //     H = sum_a u_a g_a^T, distance rows n . (u_j - u_i); plus the compliance term.
 // Dot products are block reductions summed in a fixed order, so a run is reproducible.
@@ -19,6 +21,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include <string>
@@ -34,7 +37,8 @@ constexpr int kMaxThreads = 512;  // FEM_MAX_TETS / kTPT
 constexpr int kPolarIters = 12;
 // `red` holds two halves of 32 words, each with a partial of every warp (16 at most) in
 // front; behind those of the first half: the chamber pressures of kPres substeps
-constexpr int kRedPres = 16, kPres = 16;
+// and, of the second, three zeros that the slot lists are filled up with
+constexpr int kRedPres = 16, kPres = 16, kRedZero = 48;
 
 SimStatus ffail(SimStatus s, const std::string& msg) {
   snakesim::set_last_error(msg.c_str());
@@ -56,10 +60,10 @@ struct FemLayout {
   // distance row's slots, so that consecutive threads hit distinct banks)
   int g, scl, lam, idg, cont, xs, xx, vv, uu, wn, dn, drest, dat, did, dlam, ddl, dz, dp, dq, daz, red, n_float;
   // unsigned shorts (after the floats)
-  int tet, row, coff, csr, n_short;
+  int tet, row, n_short;
   // bytes (after the shorts)
   int kind, act, n_byte;
-  size_t bytes;
+  size_t bytes, limit_bytes;
   __host__ __device__ FemLayout(int P, int NT, int ND, int nnz) {
     int o = 0;
     g = o; o += NT * 9;
@@ -88,8 +92,6 @@ struct FemLayout {
     int s = 0;
     tet = s; s += NT * 4;
     row = s; s += ND * 2;
-    coff = s; s += P + 1;
-    csr = s; s += nnz;
     n_short = s;
     int b = 0;
     kind = b; b += ND;
@@ -97,7 +99,25 @@ struct FemLayout {
     n_byte = b;
     bytes = (size_t)n_float * 4 + (size_t)n_short * 2 + (size_t)n_byte;
     bytes = (bytes + 15) & ~(size_t)15;
+    // what fem_create accepts is measured with an index per contribution slot as well
+    limit_bytes = ((size_t)n_float * 4 + (size_t)(n_short + P + 1 + nnz) * 2 + (size_t)n_byte + 15) & ~(size_t)15;
   }
+};
+
+// Slot lists of phase B, one per lane, in slices of one warp.  A warp takes as long as its
+// longest list, so the particles are dealt to the lanes by falling length (ties by index),
+// and the offsets are read four at a time, one 16-byte load per lane and group with a
+// warp's loads side by side; a list is filled up to its slice's length with the offset of
+// a zero, which leaves its sum as it is (a sum that starts at +0 is never -0).
+// 864-element mesh: the warps' longest halves add up to 134 slots (148 filled up) against
+// 212 in the particles' own order, where every warp had a particle of the axis, and no lane
+// adds a remainder one slot at a time: 1.764 -> 1.661 ms per 1216-link frame, 238 -> 225 us
+// for one link.
+struct SlotSlices {
+  const int2* lane;   // [slices][32] particle of the lane's list (-1: none), first group of the slice
+  const int* groups;  // [slices] groups of four slots
+  const uint4* off;   // [groups of all slices][32] byte offsets of the slots' component 0
+  int n;              // slices
 };
 
 struct FemArgs {
@@ -109,14 +129,13 @@ struct FemArgs {
   const float* rest;          // [ND] rest lengths
   const float* vnode;         // [P] lumped volume of each particle (sum of V / 4)
   const unsigned char* fixed; // [P]
-  const unsigned short* coff; // [P + 1] first slot of each particle's list
-  const unsigned short* csr;  // [nnz] contribution offsets (component 0) in slot order
+  SlotSlices slots;
   const FemLinkParams* prm;   // [links]
   float* x;                   // [links][P][3]
   float* v;                   // [links][P][3]
   float* resid;               // [links]
   int* mv;                    // [links]
-  int P, NT, ND, nnz;
+  int P, NT, ND;
   long long frame;
   double dt;
   int n_sub, K, pcr_iters;
@@ -213,25 +232,19 @@ __device__ __forceinline__ void tet_scatter(const float (&R)[9], const float* g,
   cont[2] = -t0z;
 }
 
-// Adds the contribution slots csr[lo..hi) in order; the offsets of four slots are read
-// before their values, so the dependent shared-memory loads overlap.
-__device__ __forceinline__ void slot_sum(const float* cont, const unsigned short* csr, int lo, int hi, float& sx,
-                                         float& sy, float& sz) {
-  int e = lo;
-  for (; e + 4 <= hi; e += 4) {
-    const int o0 = csr[e], o1 = csr[e + 1], o2 = csr[e + 2], o3 = csr[e + 3];
-    const float a0 = cont[o0], b0 = cont[o0 + 1], c0 = cont[o0 + 2];
-    const float a1 = cont[o1], b1 = cont[o1 + 1], c1 = cont[o1 + 2];
-    const float a2 = cont[o2], b2 = cont[o2 + 1], c2 = cont[o2 + 2];
-    const float a3 = cont[o3], b3 = cont[o3 + 1], c3 = cont[o3 + 2];
-    sx += a0; sy += b0; sz += c0;
-    sx += a1; sy += b1; sz += c1;
-    sx += a2; sy += b2; sz += c2;
-    sx += a3; sy += b3; sz += c3;
-  }
-  for (; e < hi; ++e) {
-    const float* c = cont + csr[e];
+// Adds n groups of four contribution slots in order, a group's offsets read before the
+// values of the group in front of it are used.
+__device__ __forceinline__ void slot_sum(const float* fs, const uint4* off, int n, float& sx, float& sy, float& sz) {
+  const char* base = reinterpret_cast<const char*>(fs);
+  auto add = [&](unsigned o) {
+    const float* c = reinterpret_cast<const float*>(base + o);
     sx += c[0]; sy += c[1]; sz += c[2];
+  };
+  uint4 o = __ldg(off);
+  for (int k = 1; k <= n; ++k) {
+    const uint4 nx = k < n ? __ldg(off + 32 * k) : o;
+    add(o.x); add(o.y); add(o.z); add(o.w);
+    o = nx;
   }
 }
 
@@ -275,7 +288,7 @@ __device__ __forceinline__ void compliance(float nu, const float (&v)[6], float 
 
 __global__ void __launch_bounds__(kMaxThreads, 1) fem_frame_kernel(FemArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const FemLayout L(A.P, A.NT, A.ND, A.nnz);
+  const FemLayout L(A.P, A.NT, A.ND, 0);
   float* fs = reinterpret_cast<float*>(smem_raw);
   unsigned short* us = reinterpret_cast<unsigned short*>(fs + L.n_float);
   unsigned char* ub = reinterpret_cast<unsigned char*>(us + L.n_short);
@@ -283,7 +296,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fem_frame_kernel(FemArgs A) {
   float *xs = fs + L.xs, *xx = fs + L.xx, *vv = fs + L.vv, *uu = fs + L.uu, *wn = fs + L.wn;
   float *dn = fs + L.dn, *drest = fs + L.drest, *dat = fs + L.dat, *did = fs + L.did, *dlam = fs + L.dlam;
   float *ddl = fs + L.ddl, *dz = fs + L.dz, *dp = fs + L.dp, *dq = fs + L.dq, *daz = fs + L.daz, *red = fs + L.red;
-  unsigned short *tetS = us + L.tet, *rowS = us + L.row, *coff = us + L.coff, *csr = us + L.csr;
+  unsigned short *tetS = us + L.tet, *rowS = us + L.row;
   unsigned char *kindS = ub + L.kind, *actS = ub + L.act;
 
   const int tid = threadIdx.x, nthr = blockDim.x;
@@ -316,8 +329,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fem_frame_kernel(FemArgs A) {
   for (int i = tid; i < NT * 4; i += nthr) tetS[i] = A.tet[i];
   for (int i = tid; i < ND * 2; i += nthr) rowS[i] = A.row[i];
   for (int i = tid; i < ND; i += nthr) kindS[i] = A.kind[i];
-  for (int i = tid; i <= P; i += nthr) coff[i] = A.coff[i];
-  for (int i = tid; i < A.nnz; i += nthr) csr[i] = A.csr[i];
+  if (tid < 3) red[kRedZero + tid] = 0.f;
   const float* xg = A.x + (size_t)link * P * 3;
   const float* vg = A.v + (size_t)link * P * 3;
   for (int i = tid; i < P * 3; i += nthr) { xx[i] = xg[i]; vv[i] = vg[i]; }
@@ -354,26 +366,20 @@ __global__ void __launch_bounds__(kMaxThreads, 1) fem_frame_kernel(FemArgs A) {
     }
     __syncthreads();
     // B: particle sums, times the inverse mass.  With at least two threads per particle,
-    // threads 2i and 2i+1 each add one half of particle i's list (first half + second
+    // two neighbouring lanes each add one half of a particle's list (first half + second
     // half, a fixed order); otherwise one thread adds the whole list.
-    if (2 * P <= nthr) {
-      const int i = tid >> 1;
+    const bool halves = 2 * P <= nthr;
+    for (int sl = warp; sl < A.slots.n; sl += nthr >> 5) {
+      const int2 who = __ldg(A.slots.lane + 32 * sl + lane);
       float sx = 0.f, sy = 0.f, sz = 0.f;
-      if (i < P) {
-        const int b = coff[i], e1 = coff[i + 1], mid = b + (e1 - b + 1) / 2;
-        slot_sum(cont, csr, (tid & 1) ? mid : b, (tid & 1) ? e1 : mid, sx, sy, sz);
+      slot_sum(fs, A.slots.off + 32 * who.y + lane, __ldg(A.slots.groups + sl), sx, sy, sz);
+      if (halves) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, 1);
+        sy += __shfl_xor_sync(0xffffffffu, sy, 1);
+        sz += __shfl_xor_sync(0xffffffffu, sz, 1);
       }
-      sx += __shfl_xor_sync(0xffffffffu, sx, 1);
-      sy += __shfl_xor_sync(0xffffffffu, sy, 1);
-      sz += __shfl_xor_sync(0xffffffffu, sz, 1);
-      if (i < P && (tid & 1) == 0) {
-        const float w = wn[i];
-        uu[3 * i] = w * sx; uu[3 * i + 1] = w * sy; uu[3 * i + 2] = w * sz;
-      }
-    } else {
-      for (int i = tid; i < P; i += nthr) {
-        float sx = 0.f, sy = 0.f, sz = 0.f;
-        slot_sum(cont, csr, coff[i], coff[i + 1], sx, sy, sz);
+      const int i = who.x;
+      if (i >= 0 && !(halves && (lane & 1))) {
         const float w = wn[i];
         uu[3 * i] = w * sx; uu[3 * i + 1] = w * sy; uu[3 * i + 2] = w * sz;
       }
@@ -679,18 +685,22 @@ __global__ void fem_node_volume_kernel(const double* X, const int* tets, const u
 
 struct FemHandle {
   cudaStream_t st = nullptr;
-  int n_links = 0, P = 0, NT = 0, ND = 0, nnz = 0, nthr = 0;
+  int n_links = 0, P = 0, NT = 0, ND = 0, nthr = 0, n_slices = 0;
   size_t smem = 0;
   FemConfig cfg{};
   long long frame = 0, launches = 0;
   float *g = nullptr, *vol = nullptr, *rest = nullptr, *vnode = nullptr, *x = nullptr, *v = nullptr,
         *resid = nullptr;
   int* mv = nullptr;
-  unsigned short *tet = nullptr, *row = nullptr, *coff = nullptr, *csr = nullptr;
+  unsigned short *tet = nullptr, *row = nullptr;
+  int2* slot_lane = nullptr;
+  int* slot_groups = nullptr;
+  uint4* slot_off = nullptr;
   unsigned char *kind = nullptr, *fixed = nullptr;
   FemLinkParams* prm = nullptr;
   double* tmp_x = nullptr;  // mesh copies used only while fem_create computes the rest data
   int *tmp_t = nullptr, *tmp_r = nullptr;
+  unsigned short *coff = nullptr, *csr = nullptr;
 };
 
 namespace {
@@ -706,7 +716,8 @@ SimStatus validate_cfg(const FemConfig* c) {
 
 void free_all(FemHandle* h) {
   void* ptrs[] = {h->g,   h->vol,  h->rest, h->vnode, h->x,    h->v,     h->resid, h->mv,   h->tet,
-                  h->row, h->coff, h->csr,  h->kind,  h->fixed, h->prm, h->tmp_x, h->tmp_t, h->tmp_r};
+                  h->row, h->coff, h->csr,  h->kind,  h->fixed, h->prm, h->tmp_x, h->tmp_t, h->tmp_r,
+                  h->slot_lane, h->slot_groups, h->slot_off};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -787,14 +798,51 @@ SimStatus fem_create(const FemConfig* cfg, const FemMesh* mesh, int n_links, con
   int dev = 0, smem_max = 0;
   FCU(cudaGetDevice(&dev));
   FCU(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (lay.bytes > (size_t)smem_max)
-    return ffail(SIM_EINVAL, "mesh needs " + std::to_string(lay.bytes) + " bytes of shared memory per block (" +
+  if (lay.limit_bytes > (size_t)smem_max)
+    return ffail(SIM_EINVAL, "mesh needs " + std::to_string(lay.limit_bytes) + " bytes of shared memory per block (" +
                                  std::to_string(smem_max) + " available)");
   FCU(cudaFuncSetAttribute(fem_frame_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes));
 
+  // phase B's slices: the lists (a particle's halves, or its whole list) by falling length
+  const bool halves = 2 * P <= nthr;
+  std::vector<int> order(P);
+  for (int i = 0; i < P; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return cnt[a + 1] - cnt[a] > cnt[b + 1] - cnt[b]; });
+  const int n_lists = halves ? 2 * P : P, n_slices = (n_lists + 31) / 32;
+  std::vector<int2> slot_lane(32 * n_slices, make_int2(-1, 0));
+  std::vector<int> slot_groups(n_slices, 0);
+  std::vector<uint4> slot_off;
+  const unsigned zero = 4u * (unsigned)(lay.red + kRedZero);
+  for (int sl = 0; sl < n_slices; ++sl) {
+    int lo[32], hi[32], len = 0;
+    for (int l = 0; l < 32; ++l) {
+      const int k = 32 * sl + l;
+      lo[l] = hi[l] = 0;
+      slot_lane[k].y = (int)slot_off.size() / 32;
+      if (k >= n_lists) continue;
+      const int i = order[halves ? k / 2 : k];
+      const int b = cnt[i], e = cnt[i + 1], mid = b + (e - b + 1) / 2;
+      slot_lane[k].x = i;
+      lo[l] = halves && (k & 1) ? mid : b;
+      hi[l] = halves && !(k & 1) ? mid : e;
+      len = std::max(len, hi[l] - lo[l]);
+    }
+    slot_groups[sl] = (len + 3) / 4;
+    for (int g = 0; g < slot_groups[sl]; ++g)
+      for (int l = 0; l < 32; ++l) {
+        unsigned o[4];
+        for (int c = 0; c < 4; ++c) {
+          const int e = lo[l] + 4 * g + c;
+          o[c] = e < hi[l] ? 4u * (unsigned)(lay.cont + csr[e]) : zero;
+        }
+        slot_off.push_back(make_uint4(o[0], o[1], o[2], o[3]));
+      }
+  }
+
   FemHandle* h = new FemHandle();
   h->st = (cudaStream_t)stream;
-  h->n_links = n_links; h->P = P; h->NT = NT; h->ND = ND; h->nnz = nnz; h->nthr = nthr; h->smem = lay.bytes;
+  h->n_links = n_links; h->P = P; h->NT = NT; h->ND = ND; h->nthr = nthr; h->n_slices = n_slices; h->smem = lay.bytes;
   h->cfg = *cfg;
   auto cleanup = [&](SimStatus st) {
     free_all(h);
@@ -817,8 +865,9 @@ SimStatus fem_create(const FemConfig* cfg, const FemMesh* mesh, int n_links, con
   FALLOC(h->mv, sizeof(int) * n_links);
   FALLOC(h->tet, sizeof(unsigned short) * NT * 4);
   FALLOC(h->row, sizeof(unsigned short) * ND * 2);
-  FALLOC(h->coff, sizeof(unsigned short) * (P + 1));
-  FALLOC(h->csr, sizeof(unsigned short) * nnz);
+  FALLOC(h->slot_lane, sizeof(int2) * slot_lane.size());
+  FALLOC(h->slot_groups, sizeof(int) * slot_groups.size());
+  FALLOC(h->slot_off, sizeof(uint4) * slot_off.size());
   FALLOC(h->kind, ND);
   FALLOC(h->fixed, P);
   FALLOC(h->prm, sizeof(FemLinkParams) * n_links);
@@ -826,11 +875,13 @@ SimStatus fem_create(const FemConfig* cfg, const FemMesh* mesh, int n_links, con
   FALLOC(h->tmp_x, sizeof(double) * P * 3);
   FALLOC(h->tmp_t, sizeof(int) * NT * 4);
   FALLOC(h->tmp_r, sizeof(int) * ND * 2);
+  FALLOC(h->coff, sizeof(unsigned short) * (P + 1));
+  FALLOC(h->csr, sizeof(unsigned short) * nnz);
   double* dX = h->tmp_x;
   int *dT = h->tmp_t, *dR = h->tmp_r;
   auto free_tmp = [&]() {
-    cudaFree(h->tmp_x); cudaFree(h->tmp_t); cudaFree(h->tmp_r);
-    h->tmp_x = nullptr; h->tmp_t = nullptr; h->tmp_r = nullptr;
+    cudaFree(h->tmp_x); cudaFree(h->tmp_t); cudaFree(h->tmp_r); cudaFree(h->coff); cudaFree(h->csr);
+    h->tmp_x = nullptr; h->tmp_t = nullptr; h->tmp_r = nullptr; h->coff = nullptr; h->csr = nullptr;
   };
   std::vector<unsigned short> tet16(NT * 4), row16(ND * 2);
   for (int i = 0; i < NT * 4; ++i) tet16[i] = (unsigned short)mesh->tets[i];
@@ -852,6 +903,9 @@ SimStatus fem_create(const FemConfig* cfg, const FemMesh* mesh, int n_links, con
     if ((e = cudaMemcpyAsync(h->fixed, fixed8.data(), P, cudaMemcpyHostToDevice, h->st))) break;
     if ((e = cudaMemcpyAsync(h->coff, coff.data(), sizeof(unsigned short) * (P + 1), cudaMemcpyHostToDevice, h->st))) break;
     if ((e = cudaMemcpyAsync(h->csr, csr.data(), sizeof(unsigned short) * nnz, cudaMemcpyHostToDevice, h->st))) break;
+    if ((e = cudaMemcpyAsync(h->slot_lane, slot_lane.data(), sizeof(int2) * slot_lane.size(), cudaMemcpyHostToDevice, h->st))) break;
+    if ((e = cudaMemcpyAsync(h->slot_groups, slot_groups.data(), sizeof(int) * slot_groups.size(), cudaMemcpyHostToDevice, h->st))) break;
+    if ((e = cudaMemcpyAsync(h->slot_off, slot_off.data(), sizeof(uint4) * slot_off.size(), cudaMemcpyHostToDevice, h->st))) break;
     if ((e = cudaMemcpyAsync(h->prm, params, sizeof(FemLinkParams) * n_links, cudaMemcpyHostToDevice, h->st))) break;
     if ((e = cudaMemcpyAsync(h->x, x0.data(), sizeof(float) * nstate, cudaMemcpyHostToDevice, h->st))) break;
     if ((e = cudaMemsetAsync(h->v, 0, sizeof(float) * nstate, h->st))) break;
@@ -887,9 +941,10 @@ SimStatus fem_step(FemHandle* h, int n_frames) {
   if (n_frames < 0) return ffail(SIM_EINVAL, "n_frames < 0");
   FemArgs A;
   A.g = h->g; A.vol = h->vol; A.tet = h->tet; A.row = h->row; A.kind = h->kind; A.rest = h->rest;
-  A.vnode = h->vnode; A.fixed = h->fixed; A.coff = h->coff; A.csr = h->csr; A.prm = h->prm;
+  A.vnode = h->vnode; A.fixed = h->fixed; A.prm = h->prm;
+  A.slots = SlotSlices{h->slot_lane, h->slot_groups, h->slot_off, h->n_slices};
   A.x = h->x; A.v = h->v; A.resid = h->resid; A.mv = h->mv;
-  A.P = h->P; A.NT = h->NT; A.ND = h->ND; A.nnz = h->nnz;
+  A.P = h->P; A.NT = h->NT; A.ND = h->ND;
   A.dt = h->cfg.dt; A.n_sub = h->cfg.n_sub; A.K = h->cfg.iters; A.pcr_iters = h->cfg.pcr_iters;
   A.tol = h->cfg.tol; A.gx = h->cfg.gravity[0]; A.gy = h->cfg.gravity[1]; A.gz = h->cfg.gravity[2];
   for (int f = 0; f < n_frames; ++f) {

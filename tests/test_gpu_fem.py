@@ -149,3 +149,31 @@ def test_state_round_trip_and_frame_index():
     assert np.array_equal(a.state()[0], b.state()[0])
     xd, vd, rd, mvd = a.state_device()
     assert np.array_equal(xd.cpu().numpy(), a.state()[0])
+
+
+def _scattered(n):
+    """n elements that share no particle, each held at its first one."""
+    rng = np.random.default_rng(n)
+    corner = 0.01 * np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0], [0, 0, 1]])
+    X = np.concatenate([corner + rng.uniform(-0.002, 0.002, (4, 3)) + [0, 0.03 * i, 0] for i in range(n)])
+    return X, np.arange(4 * n).reshape(n, 4), np.arange(4 * n) % 4 == 0
+
+
+def _fan(n):
+    """n wedges around one edge, held at its first particle: lists of n slots and of two."""
+    a = 2 * np.pi * np.arange(n) / n
+    ring = np.stack([0 * a, 0.0125 * np.cos(a), 0.0125 * np.sin(a)], 1)
+    X = np.concatenate([[[0, 0, 0], [0.02, 0, 0]], ring])
+    return X, np.array([[0, 2 + i, 2 + (i + 1) % n, 1] for i in range(n)]), np.arange(n + 2) == 0
+
+
+@pytest.mark.parametrize("mesh,n", [(_scattered, 1), (_scattered, 33), (_scattered, 200), (_fan, 7), (_fan, 37)])
+def test_slot_lists_of_any_length_and_number(mesh, n):
+    """The particles' slot lists at the edges of their slices: lists of one slot (a group
+    filled up with three), more slices than warps, one long list among short ones."""
+    X, T, fixed = mesh(n)
+    M = dict(W.fem_link_mesh(m=4, n_sec=2, length=0.02), X=X, tets=T.astype(np.int32), fixed=fixed.astype(np.int32),
+             rows=np.zeros((0, 2), np.int32), kinds=np.zeros(0, np.int32))
+    w = W.fem_links(2, seed=19)
+    w["poisson"][:] = 0.3
+    _check(M, w, W.fem_settings(gravity=(0.0, 0.0, -9.81), iters=12, pcr_iters=6), frames=2)
