@@ -22,7 +22,9 @@
  *   a7  updates velocities from the displacement with exponential damping.
  * Thousands of snakes of uneven length run together: the snakes are grouped by length
  * into lane layouts (8, 16 or 32 lanes per snake, 1-4 nodes per lane), and each layout
- * runs one persistent kernel that takes its snakes from a device-side work queue.
+ * runs one persistent kernel that takes its snakes from a device-side work queue.  Where
+ * the chip has warps to spare, the 8- and 16-lane layouts spread one snake over a whole
+ * warp, with the same results to the bit.
  *
  * Conventions (every call):
  *   - Every call returns a SimStatus; nothing aborts or throws across the ABI.  The text
@@ -243,7 +245,9 @@ SimStatus sim_snapshot_restore(SimHandle* h);
  * segment is recomputed, its substeps are walked in reverse and, inside each, the K
  * iterates are recomputed and transposed (clamps and the friction projection take the
  * derivative of the branch they took).  Working memory grows with ckpt_every x n_sub
- * substep states per snake.  Errors: SIM_EINVAL, SIM_ENOMEM, SIM_ECUDA. */
+ * substep states per snake, and sim_calib_forward keeps the substep states of the last
+ * segments besides, up to 1 GiB, where the device has room for them (the backward pass
+ * then leaves their recomputation out).  Errors: SIM_EINVAL, SIM_ENOMEM, SIM_ECUDA. */
 SimStatus sim_calib_forward(SimHandle* h, const float* theta, int n_steps, int ckpt_every,
                             float* tips);
 SimStatus sim_calib_backward(SimHandle* h, const float* tips_bar, float* grad_theta);
