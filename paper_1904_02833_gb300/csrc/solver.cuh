@@ -369,8 +369,10 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
 //  * substep-start differences, contact heights and the friction frame are formed once;
 //  * a row that does not exist has a zero in the constant its update is multiplied by (the
 //    stretch row's reciprocal weight, the contact and friction rows' omega m, an infinite
-//    bend weight) instead of selects; its segment is a straight dummy whose positions are
-//    chosen once.  Residual terms are masked by a 0 / 1 factor;
+//    bend weight) instead of selects, which needs every term of such a row finite: its
+//    segment is the straight dummy (1, 0, 0) at any displacement, the slots' difference
+//    being multiplied by 0 there (by 1, and added with the same rounding, where the segment
+//    exists).  Residual terms are masked by a 0 / 1 factor;
 //  * a pass in which every live group has a bilateral term over the tolerance (and the cap
 //    is not reached) stops nothing: it needs neither the contact and friction residuals nor
 //    the stop logic, and updates without selects.  The other passes take the second form.
@@ -389,6 +391,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
   const unsigned gm = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(unsigned)(G - 1)));
   // constants of the substep
   float xd[NPL + 1][3];         // segment vectors at the substep start, u: segment i0 + u - 1
+  float se[NPL + 1];            // 1 where that segment exists, else 0 (a dummy vector in xd)
   float w[NPL + 2];             // inverse masses of nodes i0 - 1 .. i0 + NPL
   float ws[NPL], rs[NPL];       // stretch: residual mask, omega-free reciprocal weight
   float wb[NPL], ab[NPL];       // bend: residual mask, compliance in the weight (inf: no row)
@@ -400,6 +403,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     const bool on = valid && i >= 0 && i + 1 <= S.N - 1;
     const float* a = (u == 0) ? xsl : xs[u > 0 ? u - 1 : 0];
     const float* b = (u == NPL) ? xsr : xs[u < NPL ? u : 0];
+    se[u] = on ? 1.f : 0.f;
     xd[u][0] = on ? b[0] - a[0] : 1.f;
     xd[u][1] = on ? b[1] - a[1] : 0.f;
     xd[u][2] = on ? b[2] - a[2] : 0.f;
@@ -450,7 +454,8 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     auto seg = [&](int u) {
       const float* ad = (u == 0) ? dxl : dx[u > 0 ? u - 1 : 0];
       const float* bd = (u == NPL) ? dxr : dx[u < NPL ? u : 0];
-      return make_seg(xd[u][0] + (bd[0] - ad[0]), xd[u][1] + (bd[1] - ad[1]), xd[u][2] + (bd[2] - ad[2]), L0);
+      return make_seg(fmaf(se[u], bd[0] - ad[0], xd[u][0]), fmaf(se[u], bd[1] - ad[1], xd[u][1]),
+                      fmaf(se[u], bd[2] - ad[2], xd[u][2]), L0);
     };
     float acc[NPL][3], dl[NPL][6];
     float accL[3] = {0.f, 0.f, 0.f}, accR[3] = {0.f, 0.f, 0.f};

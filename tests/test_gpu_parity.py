@@ -553,3 +553,45 @@ def test_one_snake_per_warp_gives_the_layouts_bits(lanes, npl, mode):
         assert np.array_equal(sa[k], sb[k][:len(sa[k])]), k
         assert np.array_equal(sa[k], sb[k][-len(sa[k]):]), k
     assert torch.equal(a.lam(), b.lam()[:a.n_nodes])
+
+
+@pytest.mark.parametrize("lanes,npl", [(8, 1), (8, 2), (8, 3), (8, 4), (16, 1), (16, 2), (16, 3), (16, 4),
+                                       (32, 1), (32, 2), (32, 3), (32, 4)])
+@pytest.mark.parametrize("copies", [1, 2500])
+def test_absent_segments_do_not_follow_the_displacements(lanes, npl, copies):
+    """A snake that flies one length unit along +x in a substep, and one whose first node moves
+    one unit against the others: the slots around the chain have no segment, whatever their
+    displacement differences.  Snakes with slots to spare and without, one per warp and several;
+    the flying ones keep their shape exactly (all lengths are powers of two), the torn ones
+    follow the oracle."""
+    cap = lanes * npl
+    n = sorted({2, 3, max(2, cap - npl), max(2, cap - 1), cap})
+    w = W.batched(n=2 * len(n), seed=51, links=(1, 1))
+    w["seg_per_link"][:] = np.repeat(n, 2) - 1
+    for k, v in dict(L0=1 / 64, yaw0=0.0, gait_amp=0.0, damping=0.0, z0=1.0).items():
+        w[k][:] = v
+    w = {k: np.tile(v, copies) for k, v in w.items()}
+    s = W.solver_settings(dt=0.125, n_sub=1, iters=4, gravity=(0.0, 0.0, 0.0), contact=False)
+    first = np.concatenate([[0], np.cumsum(W.n_nodes(w))])
+    vel = np.zeros((first[-1], 3), np.float32)
+    torn = np.zeros(first[-1], bool)
+    for k in range(0, len(first) - 1, 2):
+        vel[first[k]:first[k + 1], 0] = 8.0
+        vel[first[k + 1], 0] = -8.0
+        torn[first[k + 1]:first[k + 2]] = True
+    g = Sim(w, s)
+    for N in n:
+        g.set_layout(int(N), lanes, npl)
+    x0 = g.state_host()["pos"]
+    g.set_state(vel=vel)
+    g.step(1)
+    x = g.state_host()["pos"]
+    assert np.array_equal(x[~torn], x0[~torn] + np.float32([1.0, 0.0, 0.0]))
+    assert (g.state_host()["resid"][::2] == 0.0).all()
+    one = {k: v[:2 * len(n)] for k, v in w.items()}
+    o = oracle.OracleSim(one, s)
+    m = first[2 * len(n)]
+    o.v[:] = vel[:m]
+    o.step(1)
+    assert np.abs(x[:m] - o.x).max() <= 1e-5
+    assert np.array_equal(x[:m], x[-m:])
