@@ -22,9 +22,10 @@
  *   a7  updates velocities from the displacement with exponential damping.
  * Thousands of snakes of uneven length run together: the snakes are grouped by length
  * into lane layouts (8, 16 or 32 lanes per snake, 1-4 nodes per lane), and each layout
- * runs one persistent kernel that takes its snakes from a device-side work queue.  Where
- * the chip has warps to spare, the 8- and 16-lane layouts spread one snake over a whole
- * warp, with the same results to the bit.
+ * runs one persistent kernel that takes its snakes from a device-side work queue.  The 8- and
+ * 16-lane layouts spread one snake over a whole warp instead where that form measures faster
+ * (small batches, and solves to a tolerance of snakes that fill the warp's node slots), with
+ * the same results to the bit.
  *
  * Conventions (every call):
  *   - Every call returns a SimStatus; nothing aborts or throws across the ABI.  The text
@@ -209,7 +210,9 @@ SimStatus sim_get_status(SimHandle* h, int32_t* status);
 SimStatus sim_autotune(SimHandle* h, int n_steps);
 
 /* Current layout of a bucket of snakes with `nodes` nodes: lanes per snake (8, 16, 32)
- * and nodes per lane (1..4); 0 if no snake has that length. */
+ * and nodes per lane (1..4); 0 if no snake has that length.  A layout fixes the order in which
+ * a node's row contributions are added, hence the results' bits; the kernel that runs it may
+ * use more lanes for a snake. */
 SimStatus sim_get_layout(SimHandle* h, int nodes, int32_t* lanes, int32_t* nodes_per_lane);
 
 /* Forces the layout of a bucket (lanes in {8, 16, 32}, nodes_per_lane in 1..4,

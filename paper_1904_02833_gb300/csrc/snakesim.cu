@@ -259,7 +259,7 @@ struct ItemSet {
   int lay_grid[kLayouts] = {};
   int lay_launch[kLayouts] = {};      // layouts with work, most work first
   int n_lay = 0;
-  bool wide = false;                  // the 8- and 16-lane layouts run by WIDE kernels
+  bool wide[kLayouts] = {};           // layouts run by WIDE kernels
   // Every item is one snake and all of them are resident at once, in blocks of one warp: then
   // neither grouping nor order matters, and a step needs no work queue (one snake, a captured
   // env-step: 140 us with the queue's kernel and the counter's clear before the solver,
@@ -274,7 +274,7 @@ struct ItemSet {
 };
 
 struct SimHandle : ItemSet {
-  ItemSet parked;  // the other choice of `wide`, once it has been built
+  ItemSet parked;  // the items of the other stop rule, once they have been built
   int sms = 0;
   SimConfig cfg;
   int n = 0;
@@ -382,30 +382,42 @@ int solver_var(const SimHandle* h) {
   return h->aniso ? kVarAniso : kVarJacobi;
 }
 
-// Whether the snakes of the 8- and 16-lane layouts run one per warp, by the WIDE kernels (same
-// results).  A warp of several snakes shares its issue slots but walks three or four nodes
-// per lane and, to a tolerance, goes on until its slowest snake has converged.  Measured on
-// uneven snakes of 21-61 nodes (us per env-step, several per warp / one per warp): to 1e-4
-// from the previous multipliers 3245 / 1329 (one snake), 7004 / 2293 (1216), 10850 / 8045
-// (9728), 19724 / 14475 (19456), and alike from cold ones; at ten fixed updates 257 / 133
-// (one snake), 267 / 175 (1216), 334 / 339 (2432), 957 / 1047 (9728).  So: always to a
-// tolerance, and at fixed updates up to two snakes per warp slot of the chip.
-bool use_wide(const SimHandle* h) {
-  return solver_var(h) != kVarPcr && (h->cfg.tol > 0.f || h->n <= 16 * h->sms);
+// Whether the snakes of layout l run one per warp, by the WIDE kernels (same results).  One per
+// warp, a lane walks one or two nodes instead of up to four and, to a tolerance, a warp ends
+// with its snake instead of with the slowest of two or four; but the chip issues 4 / share
+// times the node slots, which counts once every warp slot is taken (8 warps per SM).
+// Measured, us per env-step, several per warp / one per warp, snakes of one length at ten fixed
+// updates and to 1e-4 from the previous multipliers:
+//   share  layout nodes | 1216 snakes          | 2432                 | 9728                  | 48640
+//   1      8x1      8   | 116 / 113, 211 / 209 | 118 / 194, 213 / 368 | 211 / 673, 399 / 1138 | 968 / 3245, 1619 / 5430
+//   2      8x2     15   | 147 / 113, 489 / 345 | 149 / 194, 490 / 622 | 367 / 673, 1151 / 1849 | 1752 / 3239, 5191 / 8488
+//   3      16x3    41   | 192 / 174, 3808 / 2255 | 261 / 351, 4745 / 2909 | 960 / 1322, 10152 / 10072 | 4657 / 6492, 43782 / 46272
+//   4      8x4     31   | 251 / 114, 3672 / 879 | 250 / 194, 3794 / 1516 | 641 / 674, 6913 / 4278 | 3084 / 3283, 26980 / 19781
+//   4      16x4    61   | 254 / 174, 8246 / 3103 | 334 / 348, 11117 / 4408 | 1262 / 1318, 20077 / 14055 | 6186 / 6457, 87130 / 64600
+// In uneven batches of several layouts at 1824 snakes the shares 2 and 3 are as fast either way
+// (6-41 nodes 265 / 217 at ten updates, 21-61 nodes 246 / 290).  So, in snakes of the batch per
+// SM: fixed updates 8, 12, 12 and 16 for the shares 1-4; to a tolerance 8, 12, 64 and any.
+bool use_wide(const SimHandle* h, int l) {
+  if (layout_lanes(l) == 32 || solver_var(h) == kVarPcr) return false;
+  const int slots = layout_lanes(l) * layout_npl(l);
+  const int share = 4 * slots / (slots <= 32 ? 32 : 64);  // quarters of the warp's node slots
+  const bool to_tol = h->cfg.tol > 0.f;
+  if (share == 4 && to_tol) return true;
+  const int per_sm = share == 1 ? 8 : share == 4 ? 16 : share == 3 && to_tol ? 64 : 12;
+  return h->n <= (long long)per_sm * h->sms;
 }
-bool lay_wide(const SimHandle* h, int l) { return h->wide && layout_lanes(l) < 32; }
 
 // The kernel that runs the items of layout l.
 SolverKernel solver_kernel(const SimHandle* h, bool split, int l) {
   const int var = solver_var(h);
-  if (lay_wide(h, l)) return kWideKernels[split ? 1 : 0][var][layout_lanes(l) * layout_npl(l) <= 32 ? 0 : 1];
+  if (h->wide[l]) return kWideKernels[split ? 1 : 0][var][layout_lanes(l) * layout_npl(l) <= 32 ? 0 : 1];
   return kSolverKernels[split ? 1 : 0][var][l];
 }
 
 SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = nullptr) {
   // (autotuning times the layouts themselves)
   static_cast<ItemSet*>(h)->release();
-  h->wide = !only_bucket && use_wide(h);
+  for (int l = 0; l < kLayouts; ++l) h->wide[l] = !only_bucket && use_wide(h, l);
   // group snakes by node count, pack 32/G snakes per warp item, biggest work first;
   // `only_bucket` restricts the items to the node counts it lists (autotuning)
   std::map<int, std::vector<int>> buckets;
@@ -419,7 +431,7 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
     if (only_bucket && !only_bucket->count(kv.first)) continue;
     const int lay = h->layout[kv.first];
     if (lay < 0) return fail(SIM_EINVAL, "snake too long for the lane layouts (max 128 nodes)");
-    const int per = lay_wide(h, lay) ? 1 : 32 / layout_lanes(lay);
+    const int per = h->wide[lay] ? 1 : 32 / layout_lanes(lay);
     for (int s : kv.second) cls[s] = (int)cls_base.size();
     cls_base.push_back((int)order.size());
     for (size_t b = 0; b < kv.second.size(); b += per) {
@@ -489,7 +501,7 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
   h->n_lay = 0;
   h->direct = its.size() <= (size_t)8 * h->sms;  // the warps that two blocks per SM leave room for
   for (int l = 0; l < kLayouts; ++l)
-    if (cnt[l] > 0 && layout_lanes(l) < 32 && !lay_wide(h, l)) h->direct = false;
+    if (cnt[l] > 0 && layout_lanes(l) < 32 && !h->wide[l]) h->direct = false;
   for (int l = 0; l < kLayouts; ++l) {
     h->lay_grid[l] = 0;
     if (cnt[l] == 0) continue;
@@ -514,10 +526,15 @@ SimStatus rebuild_items(SimHandle* h, const std::map<int, int>* only_bucket = nu
 // After a change of configuration: the set of items its rule asks for, kept from an earlier
 // use where there is one.
 SimStatus choose_items(SimHandle* h) {
-  if (use_wide(h) == h->wide) return SIM_OK;
+  auto fits = [&]() {
+    if (!h->items) return false;
+    for (int l = 0; l < kLayouts; ++l)
+      if (h->wide[l] != use_wide(h, l)) return false;
+    return true;
+  };
+  if (fits()) return SIM_OK;
   std::swap(static_cast<ItemSet&>(*h), h->parked);
-  if (h->items && h->wide == use_wide(h)) return SIM_OK;
-  return build_items(h);
+  return fits() ? SIM_OK : build_items(h);
 }
 
 SolverArgs make_args(SimHandle* h, int n_steps) {

@@ -595,3 +595,27 @@ def test_absent_segments_do_not_follow_the_displacements(lanes, npl, copies):
     o.step(1)
     assert np.abs(x[:m] - o.x).max() <= 1e-5
     assert np.array_equal(x[:m], x[-m:])
+
+
+@pytest.mark.parametrize("nodes", [8, 15])
+def test_short_snakes_to_a_tolerance_keep_sharing_warps_in_large_batches(nodes):
+    """A tolerance that is never reached makes a solve run its cap of ten updates: the work of
+    ten fixed updates, which takes as long, while one snake per warp would take four (8 nodes)
+    or two times (15 nodes) the warps.  Best of seven each."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = W.batched(n=128 * sms, seed=52, links=(1, 1))
+    w["seg_per_link"][:] = nodes - 1
+    g = Sim(w, W.solver_settings(iters=10))
+    g.step(2)
+    best = {}
+    for tol in (0.0, 1e-30) * 7:
+        g.set_config(tol=tol)
+        g.step(1)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        g.step(4)
+        b.record()
+        b.synchronize()
+        best[tol] = min(best.get(tol, 1e9), a.elapsed_time(b))
+        assert (g.state_host()["iters"] == 200).all()
+    assert best[1e-30] <= 1.5 * best[0.0], best
