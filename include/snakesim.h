@@ -205,7 +205,8 @@ SimStatus sim_device_state(SimHandle* h, void** pos4, void** vel4, void** press2
 SimStatus sim_get_status(SimHandle* h, int32_t* status);
 
 /* Chooses the lanes per snake and nodes per lane of every snake-length bucket by
- * timing candidate layouts with CUDA events (the state is restored afterwards).
+ * timing candidate layouts with CUDA events (the state is restored afterwards), each bucket
+ * alone, with the kernels that a step of the whole batch would use.
  * Runs synchronously.  Errors: SIM_EINVAL, SIM_ECUDA. */
 SimStatus sim_autotune(SimHandle* h, int n_steps);
 

@@ -415,11 +415,11 @@ SolverKernel solver_kernel(const SimHandle* h, bool split, int l) {
 }
 
 SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = nullptr) {
-  // (autotuning times the layouts themselves)
   static_cast<ItemSet*>(h)->release();
-  for (int l = 0; l < kLayouts; ++l) h->wide[l] = !only_bucket && use_wide(h, l);
+  for (int l = 0; l < kLayouts; ++l) h->wide[l] = use_wide(h, l);
   // group snakes by node count, pack 32/G snakes per warp item, biggest work first;
-  // `only_bucket` restricts the items to the node counts it lists (autotuning)
+  // `only_bucket` restricts the items to the node counts it lists (autotuning, which times
+  // them in the form that a step of the whole batch uses)
   std::map<int, std::vector<int>> buckets;
   for (int s = 0; s < h->n; ++s) buckets[h->node_off[s + 1] - h->node_off[s]].push_back(s);
   std::vector<int> order;
@@ -499,7 +499,7 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
   h->lay_first[0] = 0;
   for (int l = 0; l < kLayouts; ++l) h->lay_first[l + 1] = h->lay_first[l] + cnt[l];
   h->n_lay = 0;
-  h->direct = its.size() <= (size_t)8 * h->sms;  // the warps that two blocks per SM leave room for
+  h->direct = h->n <= 8LL * h->sms;  // the warps that two blocks per SM leave room for
   for (int l = 0; l < kLayouts; ++l)
     if (cnt[l] > 0 && layout_lanes(l) < 32 && !h->wide[l]) h->direct = false;
   for (int l = 0; l < kLayouts; ++l) {

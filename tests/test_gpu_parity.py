@@ -619,3 +619,23 @@ def test_short_snakes_to_a_tolerance_keep_sharing_warps_in_large_batches(nodes):
         best[tol] = min(best.get(tol, 1e9), a.elapsed_time(b))
         assert (g.state_host()["iters"] == 200).all()
     assert best[1e-30] <= 1.5 * best[0.0], best
+
+
+@pytest.mark.parametrize("tol", [0.0, 1e-4])
+def test_autotune_times_the_kernels_a_step_runs(tol):
+    """Every candidate layout is timed by two passes of what a step with that layout launches
+    (a small batch has no queue to rebuild in the one-snake-per-warp form, and has one where
+    snakes share warps)."""
+    w = W.batched(n=6, seed=53, links=(1, 1))
+    w["seg_per_link"][:] = 7
+    s = W.solver_settings(iters=50, tol=tol)
+    g = Sim(w, s)
+    expect = 0
+    for lanes in (8, 16, 32):
+        g.set_layout(8, lanes, 1)
+        n0 = g.launches()
+        g.step(1)
+        expect += 2 * (g.launches() - n0)
+    n0 = g.launches()
+    g.autotune(1)
+    assert g.launches() - n0 == expect
