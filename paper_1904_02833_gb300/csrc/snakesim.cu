@@ -259,6 +259,7 @@ struct ItemSet {
   int lay_grid[kLayouts] = {};
   int lay_launch[kLayouts] = {};      // layouts with work, most work first
   int n_lay = 0;
+  bool to_tol = false;                // the stop rule the items are for (use_wide)
   bool wide[kLayouts] = {};           // layouts run by WIDE kernels
   // Every item is one snake and all of them are resident at once, in blocks of one warp: then
   // neither grouping nor order matters, and a step needs no work queue (one snake, a captured
@@ -274,7 +275,7 @@ struct ItemSet {
 };
 
 struct SimHandle : ItemSet {
-  ItemSet parked;  // the items of the other stop rule, once they have been built
+  ItemSet parked;  // the items of the other stop rule where they differ, else empty
   int sms = 0;
   SimConfig cfg;
   int n = 0;
@@ -397,41 +398,39 @@ int solver_var(const SimHandle* h) {
 // In uneven batches of several layouts at 1824 snakes the shares 2 and 3 are as fast either way
 // (6-41 nodes 265 / 217 at ten updates, 21-61 nodes 246 / 290).  So, in snakes of the batch per
 // SM: fixed updates 8, 12, 12 and 16 for the shares 1-4; to a tolerance 8, 12, 64 and any.
-bool use_wide(const SimHandle* h, int l) {
+bool use_wide(const SimHandle* h, int l, bool to_tol) {
   if (layout_lanes(l) == 32 || solver_var(h) == kVarPcr) return false;
   const int slots = layout_lanes(l) * layout_npl(l);
   const int share = 4 * slots / (slots <= 32 ? 32 : 64);  // quarters of the warp's node slots
-  const bool to_tol = h->cfg.tol > 0.f;
   if (share == 4 && to_tol) return true;
   const int per_sm = share == 1 ? 8 : share == 4 ? 16 : share == 3 && to_tol ? 64 : 12;
   return h->n <= (long long)per_sm * h->sms;
 }
 
 // The kernel that runs the items of layout l.
-SolverKernel solver_kernel(const SimHandle* h, bool split, int l) {
+SolverKernel solver_kernel(const SimHandle* h, const ItemSet& I, bool split, int l) {
   const int var = solver_var(h);
-  if (h->wide[l]) return kWideKernels[split ? 1 : 0][var][layout_lanes(l) * layout_npl(l) <= 32 ? 0 : 1];
+  if (I.wide[l]) return kWideKernels[split ? 1 : 0][var][layout_lanes(l) * layout_npl(l) <= 32 ? 0 : 1];
   return kSolverKernels[split ? 1 : 0][var][l];
 }
 
-SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = nullptr) {
-  static_cast<ItemSet*>(h)->release();
-  for (int l = 0; l < kLayouts; ++l) h->wide[l] = use_wide(h, l);
-  // group snakes by node count, pack 32/G snakes per warp item, biggest work first;
-  // `only_bucket` restricts the items to the node counts it lists (autotuning, which times
-  // them in the form that a step of the whole batch uses)
-  std::map<int, std::vector<int>> buckets;
-  for (int s = 0; s < h->n; ++s) buckets[h->node_off[s + 1] - h->node_off[s]].push_back(s);
+// Work items of one stop rule into I, which is empty; `only_bucket` restricts them to the node
+// counts it lists (autotuning, which times them in the form that a step of the whole batch
+// uses).  On an error I may hold part of its buffers.
+typedef std::map<int, std::vector<int>> Buckets;  // node count -> snakes
+SimStatus build_set(const SimHandle* h, const Buckets& buckets, const std::map<int, int>* only_bucket, bool to_tol,
+                    ItemSet& I) {
+  I.to_tol = to_tol;
+  for (int l = 0; l < kLayouts; ++l) I.wide[l] = use_wide(h, l, to_tol);
+  // group snakes by node count, pack 32/G snakes per warp item, biggest work first
   std::vector<int> order;
   struct It { int off, cnt, lay; float cost; };
   std::vector<It> its;
   std::vector<int> cls(h->n, -1), cls_base;
   for (auto& kv : buckets) {
-    if (!h->layout.count(kv.first)) h->layout[kv.first] = default_layout(kv.first);
     if (only_bucket && !only_bucket->count(kv.first)) continue;
-    const int lay = h->layout[kv.first];
-    if (lay < 0) return fail(SIM_EINVAL, "snake too long for the lane layouts (max 128 nodes)");
-    const int per = h->wide[lay] ? 1 : 32 / layout_lanes(lay);
+    const int lay = h->layout.at(kv.first);
+    const int per = I.wide[lay] ? 1 : 32 / layout_lanes(lay);
     for (int s : kv.second) cls[s] = (int)cls_base.size();
     cls_base.push_back((int)order.size());
     for (size_t b = 0; b < kv.second.size(); b += per) {
@@ -454,87 +453,104 @@ SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = null
   });
   std::vector<int4> hitems(its.size());
   for (size_t i = 0; i < its.size(); ++i) hitems[i] = make_int4(its[i].off, its[i].cnt, its[i].lay, 0);
-  h->n_items = (int)hitems.size();
-  h->n_cls = (int)cls_base.size();
-  if (h->n_items > 0) {
-    CU(cudaMalloc(&h->items, hitems.size() * sizeof(int4)));
-    CU(cudaMalloc(&h->items0, items0.size() * sizeof(int4)));
-    CU(cudaMalloc(&h->order, order.size() * sizeof(int)));
-    CU(cudaMalloc(&h->sched_cls, h->n * sizeof(int)));
-    CU(cudaMalloc(&h->sched_base, cls_base.size() * sizeof(int)));
-    CU(cudaMalloc(&h->sched_hist, (cls_base.size() + kLayouts) * 256 * sizeof(int)));
-    CU(cudaMalloc(&h->sched_key, hitems.size() * sizeof(int)));
-    CU(cudaMemcpy(h->items, hitems.data(), hitems.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->items0, items0.data(), items0.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->order, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->sched_cls, cls.data(), h->n * sizeof(int), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->sched_base, cls_base.data(), cls_base.size() * sizeof(int), cudaMemcpyHostToDevice));
-  }
-  // feature offsets: layout by layout, snake by snake
-  h->feat_off.assign(h->n, 0);
-  {
-    long long cur = 0;
-    for (int l = 0; l < kLayouts; ++l) {
-      h->lay_fnode[l] = cur;
-      for (auto& kv : buckets) {
-        if (h->layout[kv.first] != l || (only_bucket && !only_bucket->count(kv.first))) continue;
-        for (int s : kv.second) { h->feat_off[s] = (int)cur; cur += kv.first; }
-      }
-    }
-    h->lay_fnode[kLayouts] = cur;
-    // snakes outside the scheduled classes keep their own rows past the end
-    for (auto& kv : buckets) {
-      if (!(only_bucket && !only_bucket->count(kv.first))) continue;
-      for (int s : kv.second) { h->feat_off[s] = (int)cur; cur += kv.first; }
-    }
-    if (h->feat_off_d) cudaFree(h->feat_off_d);
-    h->feat_off_d = nullptr;
-    CU(cudaMalloc(&h->feat_off_d, h->n * sizeof(int)));
-    CU(cudaMemcpy(h->feat_off_d, h->feat_off.data(), h->n * sizeof(int), cudaMemcpyHostToDevice));
+  I.n_items = (int)hitems.size();
+  I.n_cls = (int)cls_base.size();
+  if (I.n_items > 0) {
+    CU(cudaMalloc(&I.items, hitems.size() * sizeof(int4)));
+    CU(cudaMalloc(&I.items0, items0.size() * sizeof(int4)));
+    CU(cudaMalloc(&I.order, order.size() * sizeof(int)));
+    CU(cudaMalloc(&I.sched_cls, h->n * sizeof(int)));
+    CU(cudaMalloc(&I.sched_base, cls_base.size() * sizeof(int)));
+    CU(cudaMalloc(&I.sched_hist, (cls_base.size() + kLayouts) * 256 * sizeof(int)));
+    CU(cudaMalloc(&I.sched_key, hitems.size() * sizeof(int)));
+    CU(cudaMemcpy(I.items, hitems.data(), hitems.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(I.items0, items0.data(), items0.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(I.order, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(I.sched_cls, cls.data(), h->n * sizeof(int), cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(I.sched_base, cls_base.data(), cls_base.size() * sizeof(int), cudaMemcpyHostToDevice));
   }
   // per-layout ranges, grids, and launch order (most nodes x nodes per lane first)
   std::vector<double> work(kLayouts, 0.0);
   int cnt[kLayouts] = {};
   for (const It& it : its) { cnt[it.lay] += 1; work[it.lay] += it.cost * layout_npl(it.lay); }
-  h->lay_first[0] = 0;
-  for (int l = 0; l < kLayouts; ++l) h->lay_first[l + 1] = h->lay_first[l] + cnt[l];
-  h->n_lay = 0;
-  h->direct = h->n <= 8LL * h->sms;  // the warps that two blocks per SM leave room for
+  I.lay_first[0] = 0;
+  for (int l = 0; l < kLayouts; ++l) I.lay_first[l + 1] = I.lay_first[l] + cnt[l];
+  I.n_lay = 0;
+  I.direct = h->n <= 8LL * h->sms;  // the warps that two blocks per SM leave room for
   for (int l = 0; l < kLayouts; ++l)
-    if (cnt[l] > 0 && layout_lanes(l) < 32 && !h->wide[l]) h->direct = false;
+    if (cnt[l] > 0 && layout_lanes(l) < 32 && !I.wide[l]) I.direct = false;
   for (int l = 0; l < kLayouts; ++l) {
-    h->lay_grid[l] = 0;
+    I.lay_grid[l] = 0;
     if (cnt[l] == 0) continue;
     int per_sm = 0;
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(h, false, l), 128, 0));
-    const int need = h->direct ? cnt[l] : (cnt[l] + 3) / 4;  // four warps per block
-    h->lay_grid[l] = h->direct ? need : std::max(1, std::min(need, std::max(1, per_sm) * h->sms));
-    h->lay_launch[h->n_lay++] = l;
+    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solver_kernel(h, I, false, l), 128, 0));
+    const int need = I.direct ? cnt[l] : (cnt[l] + 3) / 4;  // four warps per block
+    I.lay_grid[l] = I.direct ? need : std::max(1, std::min(need, std::max(1, per_sm) * h->sms));
+    I.lay_launch[I.n_lay++] = l;
   }
-  std::stable_sort(h->lay_launch, h->lay_launch + h->n_lay,
+  std::stable_sort(I.lay_launch, I.lay_launch + I.n_lay,
                    [&](int a, int b) { return work[a] > work[b]; });
-  h->graph_dirty = true;
   return SIM_OK;
 }
 
-// New layouts or another solver: both sets of items are void.
-SimStatus rebuild_items(SimHandle* h, const std::map<int, int>* only_bucket = nullptr) {
-  h->parked.release();
-  return build_items(h, only_bucket);
-}
-
-// After a change of configuration: the set of items its rule asks for, kept from an earlier
-// use where there is one.
-SimStatus choose_items(SimHandle* h) {
-  auto fits = [&]() {
-    if (!h->items) return false;
-    for (int l = 0; l < kLayouts; ++l)
-      if (h->wide[l] != use_wide(h, l)) return false;
-    return true;
+// (Re)builds the items for new layouts or another solver: of the configured stop rule, and of
+// the other one where that runs a layout in the other form, so that a change of the tolerance
+// only picks a set (no allocation, no free; graphs captured before it keep their buffers).
+// On an error the handle keeps what it had.
+SimStatus build_items(SimHandle* h, const std::map<int, int>* only_bucket = nullptr) {
+  Buckets buckets;
+  for (int s = 0; s < h->n; ++s) buckets[h->node_off[s + 1] - h->node_off[s]].push_back(s);
+  bool differ = false;
+  const bool to_tol = h->cfg.tol > 0.f;
+  for (auto& kv : buckets) {
+    if (!h->layout.count(kv.first)) h->layout[kv.first] = default_layout(kv.first);
+    const int lay = h->layout[kv.first];
+    if (lay < 0) return fail(SIM_EINVAL, "snake too long for the lane layouts (max 128 nodes)");
+    differ |= use_wide(h, lay, true) != use_wide(h, lay, false);
+  }
+  ItemSet now, other;
+  int* feat_off_d = nullptr;
+  // feature offsets: layout by layout, snake by snake
+  std::vector<int> feat_off(h->n, 0);
+  long long lay_fnode[kLayouts + 1], cur = 0;
+  for (int l = 0; l < kLayouts; ++l) {
+    lay_fnode[l] = cur;
+    for (auto& kv : buckets) {
+      if (h->layout[kv.first] != l || (only_bucket && !only_bucket->count(kv.first))) continue;
+      for (int s : kv.second) { feat_off[s] = (int)cur; cur += kv.first; }
+    }
+  }
+  lay_fnode[kLayouts] = cur;
+  // snakes outside the scheduled classes keep their own rows past the end
+  for (auto& kv : buckets) {
+    if (!(only_bucket && !only_bucket->count(kv.first))) continue;
+    for (int s : kv.second) { feat_off[s] = (int)cur; cur += kv.first; }
+  }
+  auto build = [&]() -> SimStatus {
+    SimStatus st = build_set(h, buckets, only_bucket, to_tol, now);
+    if (st == SIM_OK && differ && !only_bucket) st = build_set(h, buckets, nullptr, !to_tol, other);
+    if (st != SIM_OK) return st;
+    CU(cudaMalloc(&feat_off_d, h->n * sizeof(int)));
+    CU(cudaMemcpy(feat_off_d, feat_off.data(), h->n * sizeof(int), cudaMemcpyHostToDevice));
+    return SIM_OK;
   };
-  if (fits()) return SIM_OK;
-  std::swap(static_cast<ItemSet&>(*h), h->parked);
-  return fits() ? SIM_OK : build_items(h);
+  const SimStatus st = build();
+  if (st != SIM_OK) {
+    now.release();
+    other.release();
+    if (feat_off_d) cudaFree(feat_off_d);
+    return st;
+  }
+  static_cast<ItemSet*>(h)->release();
+  h->parked.release();
+  if (h->feat_off_d) cudaFree(h->feat_off_d);
+  static_cast<ItemSet&>(*h) = now;
+  h->parked = other;
+  h->feat_off_d = feat_off_d;
+  h->feat_off.swap(feat_off);
+  std::copy(lay_fnode, lay_fnode + kLayouts + 1, h->lay_fnode);
+  h->graph_dirty = true;
+  return SIM_OK;
 }
 
 SolverArgs make_args(SimHandle* h, int n_steps) {
@@ -685,7 +701,7 @@ SimStatus launch_layout(SimHandle* h, const SolverArgs& A, int l, cudaStream_t s
     CU(cudaEventCreate(&tm.b));
     CU(cudaEventRecord(tm.a, s));
   }
-  solver_kernel(h, A.split != 0, l)<<<h->lay_grid[l], h->direct ? 32 : 128, 0, s>>>(B);
+  solver_kernel(h, *h, A.split != 0, l)<<<h->lay_grid[l], h->direct ? 32 : 128, 0, s>>>(B);
   CU(cudaGetLastError());
   if (timed) {
     CU(cudaEventRecord(tm.b, s));
@@ -856,10 +872,16 @@ SimStatus sim_set_config(SimHandle* h, const SimConfig* cfg) {
   if (!h) return fail(SIM_EINVAL, "null handle");
   SimStatus st = validate_cfg(cfg);
   if (st != SIM_OK) return st;
-  const bool regrid = cfg->solver != h->cfg.solver;  // another kernel variant, other occupancy
+  const SimConfig before = h->cfg;
   h->cfg = *cfg;
+  if (cfg->solver != before.solver) {  // another kernel variant, other occupancy
+    st = build_items(h);
+    if (st != SIM_OK) { h->cfg = before; return st; }
+  } else if (h->parked.items && h->to_tol != (cfg->tol > 0.f)) {
+    std::swap(static_cast<ItemSet&>(*h), h->parked);
+  }
   h->graph_dirty = true;
-  return regrid ? rebuild_items(h) : choose_items(h);
+  return SIM_OK;
 }
 
 SimStatus sim_set_pressure(SimHandle* h, const float* u, int is_device) {
@@ -1036,8 +1058,11 @@ SimStatus sim_set_layout(SimHandle* h, int nodes, int lanes, int npl) {
   if (!h) return fail(SIM_EINVAL, "null handle");
   if (!(lanes == 8 || lanes == 16 || lanes == 32) || npl < 1 || npl > 4 || lanes * npl < nodes)
     return fail(SIM_EINVAL, "layout needs lanes in {8,16,32}, nodes_per_lane in 1..4, lanes*npl >= nodes");
+  const std::map<int, int> before = h->layout;
   h->layout[nodes] = layout_id(lanes, npl);
-  return rebuild_items(h);
+  const SimStatus st = build_items(h);
+  if (st != SIM_OK) h->layout = before;
+  return st;
 }
 
 SimStatus sim_autotune(SimHandle* h, int n_steps) {
@@ -1097,7 +1122,7 @@ SimStatus sim_autotune(SimHandle* h, int n_steps) {
         one[N] = layout_id(G, npl);
         h->layout = layout0;
         h->layout[N] = layout_id(G, npl);
-        if ((st = rebuild_items(h, &one)) != SIM_OK) break;
+        if ((st = build_items(h, &one)) != SIM_OK) break;
         float ms = 0.f;
         for (int rep = 0; rep < 2 && st == SIM_OK; ++rep) {
           if (!xfer(false) || !ok(cudaEventRecord(a, h->stream), "cudaEventRecord")) break;
@@ -1121,7 +1146,7 @@ SimStatus sim_autotune(SimHandle* h, int n_steps) {
   for (void* q : {(void*)p0, (void*)v0, (void*)pr0, (void*)l0, (void*)r0, (void*)i0, (void*)s0})
     if (q) cudaFree(q);
   h->layout = run == SIM_OK ? best : layout0;
-  const SimStatus rebuilt = rebuild_items(h);
+  const SimStatus rebuilt = build_items(h);
   if (run != SIM_OK) return run;
   if (put_back != SIM_OK) return put_back;
   return rebuilt;

@@ -639,3 +639,41 @@ def test_autotune_times_the_kernels_a_step_runs(tol):
     n0 = g.launches()
     g.autotune(1)
     assert g.launches() - n0 == expect
+
+
+@pytest.mark.parametrize("learned", [False, True])
+def test_tolerance_changes_inside_a_capture_and_earlier_captures_stay_valid(learned):
+    """sim_set_config makes no CUDA call for a change of the tolerance, also where that changes
+    the kernel form of a layout (31 nodes, 8 x 4, more than 16 snakes per SM: several per warp
+    at fixed updates, one per warp to a tolerance): a step captured before the change, the
+    change and a step after it inside another capture replay what eager calls compute."""
+    from paper_1904_02833_gb300.mlp import WarmStartMLP, init_params
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = W.batched(n=17 * sms, seed=54, links=(3, 3))
+    s = W.solver_settings(iters=10, warm=2 if learned else 1, beta=0.75, net_every=7)
+    net = WarmStartMLP((0.05 * init_params(3)).astype(np.float32))
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        a, b = Sim(w, s), Sim(w, s)
+        for g in (a, b):
+            assert g.layout(31) == (8, 4)
+            g.set_mlp(net)
+            g.step(1)
+        first, second = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(first, stream=stream):
+            a.step(1)
+        with torch.cuda.graph(second, stream=stream):
+            a.set_config(tol=1e-3, iters=60)
+            a.step(1)
+        first.replay()
+        second.replay()
+        b.step(1)
+        b.set_config(tol=1e-3, iters=60)
+        b.step(1)
+        b.set_config(tol=0.0, iters=10)
+        first.replay()
+        b.step(1)
+        sa, sb = a.state_host(), b.state_host()
+    for k in ("pos", "vel", "press", "resid", "iters"):
+        assert np.array_equal(sa[k], sb[k]), k
