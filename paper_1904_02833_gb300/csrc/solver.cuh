@@ -370,9 +370,9 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
 //  * a row that does not exist has a zero in the constant its update is multiplied by (the
 //    stretch row's reciprocal weight, the contact and friction rows' omega m, an infinite
 //    bend weight) instead of selects, which needs every term of such a row finite: its
-//    segment is the straight dummy (1, 0, 0) at any displacement, the slots' difference
-//    being multiplied by 0 there (by 1, and added with the same rounding, where the segment
-//    exists).  Residual terms are masked by a 0 / 1 factor;
+//    segment is a straight dummy so long (kDummy) that no displacement of its two slots,
+//    which is added to it like to the others, can shorten it to nothing, and so short that
+//    products of two of them stay finite.  Residual terms are masked by a 0 / 1 factor;
 //  * a pass in which every live group has a bilateral term over the tolerance (and the cap
 //    is not reached) stops nothing: it needs neither the contact and friction residuals nor
 //    the stop logic, and updates without selects.  The other passes take the second form.
@@ -380,6 +380,7 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
 // form, same bits: one 41-node snake at ten updates 256 -> 200 us per env-step, 4096 uneven
 // snakes 785 -> 600 us; 8192 snakes to 1e-4 cold 49-58 -> 32-35 ms, 256 cantilevers to 1e-6
 // 30.9 -> 18.8 ms.
+constexpr float kDummy = 1.152921504606846976e18f;  // 2^60: its square is 2^120
 template <int NPL, int G, bool ANISO, bool WIDE>
 __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int q, bool valid,
                                        const float (&xs)[NPL][3], float (&dx)[NPL][3], const float (&xsl)[3],
@@ -391,7 +392,6 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
   const unsigned gm = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(unsigned)(G - 1)));
   // constants of the substep
   float xd[NPL + 1][3];         // segment vectors at the substep start, u: segment i0 + u - 1
-  float se[NPL + 1];            // 1 where that segment exists, else 0 (a dummy vector in xd)
   float w[NPL + 2];             // inverse masses of nodes i0 - 1 .. i0 + NPL
   float ws[NPL], rs[NPL];       // stretch: residual mask, omega-free reciprocal weight
   float wb[NPL], ab[NPL];       // bend: residual mask, compliance in the weight (inf: no row)
@@ -403,8 +403,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     const bool on = valid && i >= 0 && i + 1 <= S.N - 1;
     const float* a = (u == 0) ? xsl : xs[u > 0 ? u - 1 : 0];
     const float* b = (u == NPL) ? xsr : xs[u < NPL ? u : 0];
-    se[u] = on ? 1.f : 0.f;
-    xd[u][0] = on ? b[0] - a[0] : 1.f;
+    xd[u][0] = on ? b[0] - a[0] : kDummy;
     xd[u][1] = on ? b[1] - a[1] : 0.f;
     xd[u][2] = on ? b[2] - a[2] : 0.f;
   }
@@ -454,8 +453,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     auto seg = [&](int u) {
       const float* ad = (u == 0) ? dxl : dx[u > 0 ? u - 1 : 0];
       const float* bd = (u == NPL) ? dxr : dx[u < NPL ? u : 0];
-      return make_seg(fmaf(se[u], bd[0] - ad[0], xd[u][0]), fmaf(se[u], bd[1] - ad[1], xd[u][1]),
-                      fmaf(se[u], bd[2] - ad[2], xd[u][2]), L0);
+      return make_seg(xd[u][0] + (bd[0] - ad[0]), xd[u][1] + (bd[1] - ad[1]), xd[u][2] + (bd[2] - ad[2]), L0);
     };
     float acc[NPL][3], dl[NPL][6];
     float accL[3] = {0.f, 0.f, 0.f}, accR[3] = {0.f, 0.f, 0.f};
