@@ -981,7 +981,7 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid) {
     const double tp = (double)(law ? gsub + A.law_every : gsub + 1) * A.h_d;
     double cyc = (double)P.gait_freq * tp;
     cyc -= floor(cyc);
-    const float phase = 6.283185307179586f * (float)cyc;
+    const float phase = __fmul_rn(6.283185307179586f, (float)cyc);
 #pragma unroll
     for (int j = 0; j < NPL; ++j) {
       const int i = q * NPL + j;
@@ -992,12 +992,12 @@ __device__ void run_group(const SolverArgs& A, int snake, bool valid) {
         if (A.ucmd) {
           u = A.ucmd[S.lb + kl];
         } else {
-          // argument reduced to [-pi, pi] first, where the fast sine is accurate to ~1e-6
-          // (rounded as in the layout's own kernel: with one node per lane the phase's product
-          // is the fused one)
-          float arg = !WIDE ? phase + (float)kl * P.gait_lag
-                            : (A.order_npl > 1 ? fmaf((float)kl, P.gait_lag, phase)
-                                               : fmaf(6.283185307179586f, (float)cyc, (float)kl * P.gait_lag));
+          // argument reduced to [-pi, pi] first, where the fast sine is accurate to ~1e-6; the
+          // roundings of its sum are written out, so that every kernel of a layout takes the
+          // same ones (the phase's product is the fused one in the layouts of one node per lane)
+          float arg = (WIDE ? A.order_npl : NPL) > 1
+                          ? fmaf((float)kl, P.gait_lag, phase)
+                          : fmaf(6.283185307179586f, (float)cyc, __fmul_rn((float)kl, P.gait_lag));
           arg -= 6.283185307179586f * rintf(arg * 0.15915494309189535f);
           float a = P.gait_offset + P.gait_scale * __sinf(arg);
           a = fminf(1.f, fmaxf(-1.f, a)) * P.gait_amp;

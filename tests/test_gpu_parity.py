@@ -677,3 +677,44 @@ def test_tolerance_changes_inside_a_capture_and_earlier_captures_stay_valid(lear
         sa, sb = a.state_host(), b.state_host()
     for k in ("pos", "vel", "press", "resid", "iters"):
         assert np.array_equal(sa[k], sb[k]), k
+
+
+@pytest.mark.parametrize("lanes,npl", [(8, 1), (8, 2), (8, 3), (8, 4), (16, 1), (16, 2), (16, 3), (16, 4)])
+@pytest.mark.parametrize("mode", ["fixed", "tolerance", "learned", "law"])
+def test_forms_of_a_layout_agree_on_several_links_and_to_a_tolerance(lanes, npl, mode):
+    """One snake per warp (a small batch) and several (a batch beyond the chip's warps) give the
+    same bits with a phase lag between links, the chamber law, held nodes, the learned warm
+    start with its features, and to a tolerance in the layouts that run packed there."""
+    cap = lanes * npl
+    links = sorted({1, 2, 3, min(5, cap - 1), cap - 1})
+    w = W.batched(n=len(links), seed=55, links=(1, 1))
+    w["n_links"][:] = links
+    w["seg_per_link"][:] = [max(1, (cap - 1) // k) for k in links]
+    w["n_fixed"][:] = np.arange(len(links)) % 3
+    w["gait_alternate"][:] = np.arange(len(links)) % 2
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    big = {k: np.tile(v, 65 * sms // len(links) + 1) for k, v in w.items()}
+    s = W.solver_settings(iters=60 if mode == "tolerance" else 10, tol=1e-3 if mode == "tolerance" else 0.0,
+                          warm=2 if mode == "learned" else 1, beta=0.75, net_every=3, net_rows=1,
+                          latency=1 if mode == "law" else 0)
+    out = []
+    for p in (w, big):
+        g = Sim(p, s)
+        for N in np.unique(W.n_nodes(w)):
+            g.set_layout(int(N), lanes, npl)
+        if mode == "learned":
+            from paper_1904_02833_gb300.mlp import WarmStartMLP, init_params
+            g.set_mlp(WarmStartMLP((0.05 * init_params(3)).astype(np.float32)))
+        g.step_index = 41
+        g.step(3)
+        st = g.state_host()
+        n, k = int(W.n_nodes(w).sum()), len(links)
+        rec = [st["pos"][:n], st["vel"][:n], st["press"][:w["n_links"].sum()], st["resid"][:k], st["iters"][:k],
+               g.lam()[:n].cpu().numpy()]
+        if mode == "learned":
+            g.split_begin()
+            rec.append(g.features()[:6 * n].float().cpu().numpy())
+        out.append(rec)
+        g.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
