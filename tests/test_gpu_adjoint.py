@@ -165,3 +165,35 @@ def test_gradient_at_warp_edges_and_off_chip_iterates(iters):
     _, g_o = og.calib_grad(steps, target)
     for k in range(5):
         assert np.abs(g[:, k] - g_o[:, k]).max() <= 2e-2 * np.abs(g_o[:, k]).max(), (k, g[:, k], g_o[:, k])
+
+
+@pytest.mark.parametrize("contact", [False, True])
+def test_gradient_of_vertical_two_node_snakes(contact):
+    """Two nodes have no bend row, so a segment that stands straight up or hangs straight down
+    (no heading, no gradient of its elevation) is differentiable: free and held ones, and one
+    that lies flat, against the oracle's dual-number gradient.  In free flight and on a
+    contact the only parameter they depend on is the damping."""
+    from paper_1904_02833_gb300.calib import rollout, theta_of
+    from paper_1904_02833_gb300.sim import SnakeSim
+    steps = 4
+    w = {k: np.repeat(v, 4) for k, v in W.pendulum(0.125).items()}
+    w["damping"][:] = [0.1, 0.2, 0.3, 0.4]
+    w["n_fixed"][:] = [1, 0, 0, 1]
+    s = W.solver_settings(iters=10, contact=contact)
+    o = oracle.OracleSim(w, s)
+    o.x[:] = np.float32([[0, 0, 1], [0, 0, 0.9], [0, 0, 0.4], [0, 0, 0.28], [0.5, 0, 0.5], [0.5, 0, 0.625],
+                         [0, 0, 1], [0.125, 0, 1]])
+    o.v[:] = np.float32([[0, 0, 0], [0, 0, 0], [0, 0, 0.5], [0, 0, 0.25], [0.25, 0, 0], [0.25, 0, 0],
+                         [0, 0, 0], [0, 0, 0]])
+    sim = SnakeSim(w, s)
+    sim.set_state(pos=o.x.astype(np.float32), vel=o.v.astype(np.float32))
+    target = np.zeros((steps, 4, 3))
+    th = theta_of(w).cuda().requires_grad_(True)
+    tips = rollout(sim, th, steps, 2)
+    ((tips - torch.tensor(target, dtype=torch.float32, device="cuda")) ** 2).sum(-1).mean(0).sum().backward()
+    loss_o, g_o = o.calib_grad(steps, target)
+    tips_o = o.step(steps, tip=True)
+    assert np.abs(tips.detach().cpu().numpy() - tips_o).max() < 1e-4
+    g = th.grad.cpu().numpy()
+    assert np.array_equal(g[:, [0, 2, 3, 4]], np.zeros((4, 4)))
+    assert np.abs(g[:, 1] - g_o[:, 1]).max() <= 2e-2 * np.abs(g_o[:, 1]).max(), (g, g_o)
