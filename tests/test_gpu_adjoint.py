@@ -197,3 +197,57 @@ def test_gradient_of_vertical_two_node_snakes(contact):
     g = th.grad.cpu().numpy()
     assert np.array_equal(g[:, [0, 2, 3, 4]], np.zeros((4, 4)))
     assert np.abs(g[:, 1] - g_o[:, 1]).max() <= 2e-2 * np.abs(g_o[:, 1]).max(), (g, g_o)
+
+
+@pytest.mark.parametrize("rho", [2e-10, 1e-20])
+def test_nearly_vertical_segments(rho):
+    """A falling chain whose segments stand `rho` off the vertical: their fourth power (2e-10)
+    or square (1e-20) is below the smallest normal number, where the gradient's (2e-10) and
+    the forward pass's quotients still have values.  The chain falls as it stands, so the
+    gradient is the damping's alone."""
+    from paper_1904_02833_gb300.calib import rollout, theta_of
+    from paper_1904_02833_gb300.sim import SnakeSim
+    steps, N = 3, 5
+    w = W.pendulum(1 / 64)
+    w["seg_per_link"][:], w["n_fixed"][:], w["damping"][:] = N - 1, 0, 0.2
+    s = W.solver_settings(iters=6, contact=False)
+    x = np.float32(np.stack([rho * np.arange(N), np.zeros(N), 1 - np.arange(N) / 64], 1))
+    o = oracle.OracleSim(w, s)
+    o.x[:] = x
+    sim = SnakeSim(w, s)
+    sim.set_state(pos=x, vel=np.zeros((N, 3), np.float32))
+    target = np.zeros((steps, 1, 3))
+    th = theta_of(w).cuda().requires_grad_(True)
+    tips = rollout(sim, th, steps, 2)
+    g, = torch.autograd.grad((tips ** 2).sum(-1).mean(0).sum(), th)
+    _, g_o = o.calib_grad(steps, target)
+    assert np.abs(tips.detach().cpu().numpy() - o.step(steps, tip=True)).max() < 1e-5
+    if rho > 1e-12:
+        g = g.cpu().numpy()
+        assert np.isfinite(g).all(), g
+        assert abs(g[0, 1] - g_o[0, 1]) <= 2e-2 * abs(g_o[0, 1]), (g, g_o)
+
+
+def test_gradient_of_micrometre_snakes():
+    """Segments of 2^-22 m (a quarter of a micrometre; their sixth power is a subnormal number)
+    with compliances and gains that bend them like the usual ones, weightless, against the
+    oracle's dual-number gradient."""
+    from paper_1904_02833_gb300.calib import rollout, theta_of
+    from paper_1904_02833_gb300.sim import SnakeSim
+    steps, n = 4, 6
+    _, w = W.calibration(n=n, seed=12)
+    w["gain"][:] *= w["L0"] * 2.0 ** 22
+    w["L0"][:] = 2.0 ** -22
+    w["z0"][:] = 0.0
+    s = W.solver_settings(iters=6, contact=False, gravity=(0.0, 0.0, 0.0))
+    sim = SnakeSim(w, s)
+    th = theta_of(w).cuda().requires_grad_(True)
+    tips = rollout(sim, th, steps, 2)
+    scale = 1e10  # a loss of order one
+    g, = torch.autograd.grad(((scale * tips) ** 2).sum(-1).mean(0).sum(), th)
+    g = g.cpu().numpy()
+    o = oracle.OracleSim(w, s)
+    _, g_o = o.calib_grad(steps, np.zeros((steps, n, 3)))
+    g_o *= scale ** 2
+    for k in range(5):
+        assert np.abs(g[:, k] - g_o[:, k]).max() <= 2e-2 * np.abs(g_o[:, k]).max(), (k, g[:, k], g_o[:, k])
