@@ -1306,7 +1306,7 @@ SimStatus sim_calib_forward(SimHandle* h, const float* theta, int n_steps, int c
   st = advance(h, n_steps, h->stream);
   if (st != SIM_OK) return st;
   h->step_index += n_steps;
-  h->launches += 2 + 2 * ((n_steps + ckpt_every - 1) / ckpt_every);
+  h->launches += 2 + 2 * (n_steps / ckpt_every + (n_steps % ckpt_every != 0));
   return SIM_OK;
 }
 

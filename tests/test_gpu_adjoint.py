@@ -251,3 +251,15 @@ def test_gradient_of_micrometre_snakes():
     g_o *= scale ** 2
     for k in range(5):
         assert np.abs(g[:, k] - g_o[:, k]).max() <= 2e-2 * np.abs(g_o[:, k]).max(), (k, g[:, k], g_o[:, k])
+
+
+def test_checkpoint_interval_beyond_the_rollout():
+    """A checkpoint interval longer than the rollout is one segment of the rollout's length,
+    also where its substeps are more than an int counts (214748365 x 20 = 4 modulo 2^32): the
+    same tips and gradient, and no more memory than the rollout takes."""
+    steps = 3
+    _, guess, s, target, theta = setup_case(4, True, steps)
+    _, g, t = gpu_grad(guess, s, target, theta, steps, ckpt=steps)
+    for ckpt in (steps + 1, 100, 214748365, 2 ** 31 - 1):
+        _, g1, t1 = gpu_grad(guess, s, target, theta, steps, ckpt=ckpt)
+        assert np.array_equal(t, t1) and np.array_equal(g, g1), ckpt
