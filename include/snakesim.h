@@ -249,10 +249,16 @@ SimStatus sim_snapshot_restore(SimHandle* h);
  * segment is recomputed, its substeps are walked in reverse and, inside each, the K
  * iterates are recomputed and transposed (clamps and the friction projection take the
  * derivative of the branch they took).  Working memory grows with ckpt_every x n_sub
- * substep states per snake, and sim_calib_forward keeps the substep states of the last
- * segments besides, up to 1 GiB, where the device has room for them (the backward pass
- * then leaves their recomputation out).  Errors: SIM_EINVAL, SIM_ENOMEM, SIM_ECUDA. */
+ * substep states per snake (one segment of them is taken by the backward pass and kept
+ * until the handle is destroyed).  sim_calib_forward keeps the substep states of as many
+ * trailing segments as fit into 1 GiB, where the device has room for them (the backward
+ * pass then leaves their recomputation out); none where one segment is larger.
+ * sim_calib_rollout is the same rollout for callers that will hardly ask for the gradient:
+ * it keeps the checkpoints alone, and a backward pass recomputes every segment.
+ * Errors: SIM_EINVAL, SIM_ENOMEM, SIM_ECUDA. */
 SimStatus sim_calib_forward(SimHandle* h, const float* theta, int n_steps, int ckpt_every,
+                            float* tips);
+SimStatus sim_calib_rollout(SimHandle* h, const float* theta, int n_steps, int ckpt_every,
                             float* tips);
 SimStatus sim_calib_backward(SimHandle* h, const float* tips_bar, float* grad_theta);
 

@@ -22,10 +22,11 @@ def _p(t):
 
 class SnakeRollout(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, theta, sim, n_steps, ckpt_every):
+    def forward(ctx, theta, sim, n_steps, ckpt_every, grad=True):
         theta = theta.detach().to(device=sim.device, dtype=torch.float32).contiguous()
         tips = torch.empty(n_steps, sim.n, 3, device=sim.device, dtype=torch.float32)
-        N.check(sim.lib.sim_calib_forward(sim.h, _p(theta), int(n_steps), int(ckpt_every), _p(tips)))
+        run = sim.lib.sim_calib_forward if grad else sim.lib.sim_calib_rollout
+        N.check(run(sim.h, _p(theta), int(n_steps), int(ckpt_every), _p(tips)))
         ctx.sim = sim
         return tips
 
@@ -35,12 +36,13 @@ class SnakeRollout(torch.autograd.Function):
         tb = tips_bar.to(dtype=torch.float32).contiguous()
         grad = torch.empty(sim.n, 5, device=sim.device, dtype=torch.float32)
         N.check(sim.lib.sim_calib_backward(sim.h, _p(tb), _p(grad)))
-        return grad, None, None, None
+        return (grad,) + (None,) * (len(ctx.needs_input_grad) - 1)
 
 
 def rollout(sim, theta: torch.Tensor, n_steps: int, ckpt_every: int = 20) -> torch.Tensor:
-    """Tips [n_steps, n_snakes, 3] of a differentiable rollout from sim's current state."""
-    return SnakeRollout.apply(theta, sim, n_steps, ckpt_every)
+    """Tips [n_steps, n_snakes, 3] of a differentiable rollout from sim's current state (without
+    the records of the backward pass where no gradient can be asked for)."""
+    return SnakeRollout.apply(theta, sim, n_steps, ckpt_every, torch.is_grad_enabled() and theta.requires_grad)
 
 
 def theta_of(w: dict) -> torch.Tensor:

@@ -98,7 +98,7 @@ SimStatus calib_forward(CalibState& C, const SnakeParams* prm, const int* node_o
                         int n_snakes, int n_max, int l_max, const float* theta, int n_steps, int ckpt,
                         long long step0, int n_sub, int K, int contact, double dt, float omega,
                         const float* gvec, float4* pos4, float4* vel4, float2* press2, float* tips,
-                        cudaStream_t st, std::string& err);
+                        bool records, cudaStream_t st, std::string& err);
 SimStatus calib_backward(CalibState& C, const SnakeParams* prm, const float* tips_bar, float* grad, cudaStream_t st, std::string& err);
 
 // Records the message returned by sim_last_error() on this thread.

@@ -1288,7 +1288,7 @@ SimStatus sim_snapshot_restore(SimHandle* h) {
   return SIM_OK;
 }
 
-SimStatus sim_calib_forward(SimHandle* h, const float* theta, int n_steps, int ckpt_every, float* tips) {
+static SimStatus calib_run(SimHandle* h, const float* theta, int n_steps, int ckpt_every, float* tips, bool records) {
   if (!h || !theta || !tips) return fail(SIM_EINVAL, "null handle or buffer");
   if (n_steps < 1 || ckpt_every < 1) return fail(SIM_EINVAL, "n_steps and ckpt_every must be >= 1");
   if (h->cur_sub >= 0) return fail(SIM_EINVAL, "a split env-step is in progress (sim_split_finish)");
@@ -1301,13 +1301,21 @@ SimStatus sim_calib_forward(SimHandle* h, const float* theta, int n_steps, int c
   SimStatus st = calib_forward(*h->calib, h->prm, h->node_off_d, h->link_off_d, h->n, h->max_nodes,
                                h->max_links, theta, n_steps, ckpt_every, h->step_index, h->cfg.n_sub,
                                h->cfg.iters, h->cfg.contact, h->cfg.dt, h->cfg.omega, h->cfg.gravity,
-                               h->pos, h->vel, h->press, tips, h->stream, err);
+                               h->pos, h->vel, h->press, tips, records, h->stream, err);
   if (st != SIM_OK) return fail(st, err);
   st = advance(h, n_steps, h->stream);
   if (st != SIM_OK) return st;
   h->step_index += n_steps;
   h->launches += 2 + 2 * (n_steps / ckpt_every + (n_steps % ckpt_every != 0));
   return SIM_OK;
+}
+
+SimStatus sim_calib_forward(SimHandle* h, const float* theta, int n_steps, int ckpt_every, float* tips) {
+  return calib_run(h, theta, n_steps, ckpt_every, tips, true);
+}
+
+SimStatus sim_calib_rollout(SimHandle* h, const float* theta, int n_steps, int ckpt_every, float* tips) {
+  return calib_run(h, theta, n_steps, ckpt_every, tips, false);
 }
 
 SimStatus sim_calib_backward(SimHandle* h, const float* tips_bar, float* grad_theta) {

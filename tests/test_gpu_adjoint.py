@@ -263,3 +263,29 @@ def test_checkpoint_interval_beyond_the_rollout():
     for ckpt in (steps + 1, 100, 214748365, 2 ** 31 - 1):
         _, g1, t1 = gpu_grad(guess, s, target, theta, steps, ckpt=ckpt)
         assert np.array_equal(t, t1) and np.array_equal(g, g1), ckpt
+
+
+@pytest.mark.parametrize("n,steps,grad", [(512, 20, False), (4096, 14, True)])
+def test_rollouts_take_no_records_without_a_gradient_or_beyond_a_gibibyte(n, steps, grad):
+    """A rollout no gradient can be asked for (200 MB of substep states), and one whose single
+    segment's states exceed 1 GiB, take the device memory of their states and checkpoints alone
+    (here below 64 MB); the gradient of either form is the one of short segments."""
+    from paper_1904_02833_gb300.calib import rollout, theta_of
+    from paper_1904_02833_gb300.sim import SnakeSim
+    _, guess = W.calibration(n=n, seed=6)
+    s = W.solver_settings(iters=2)
+    assert n * steps * s["n_sub"] * (6 * 41 + 2 * 4) * 4 > (2 ** 30 if grad else 2e8)
+    sim, ref = SnakeSim(guess, s), SnakeSim(guess, s)
+    th = theta_of(guess).cuda().requires_grad_(grad)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    tips = rollout(sim, th, steps, steps)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 64e6
+    th2 = th.detach().clone().requires_grad_(True)
+    tips2 = rollout(ref, th2, steps, 2)
+    assert torch.equal(tips.detach(), tips2.detach())
+    if grad:
+        g, = torch.autograd.grad((tips ** 2).sum(), th)
+        g2, = torch.autograd.grad((tips2 ** 2).sum(), th2)
+        assert torch.allclose(g, g2, rtol=1e-4, atol=1e-5 * g2.abs().max().item())
