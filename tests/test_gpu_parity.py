@@ -718,3 +718,30 @@ def test_forms_of_a_layout_agree_on_several_links_and_to_a_tolerance(lanes, npl,
         g.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("solver", [0, 1])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_right_angles_whose_tangent_overflows(solver, sign):
+    """Bends of 90 degrees to within 2.5e-39: the quotient of their atan2 is infinite (lengths in
+    millimetres: 400 / 1e-36), the angle is pi / 2, and the step is the oracle's."""
+    w = W.batched(n=3, seed=56, links=(1, 1))
+    w["seg_per_link"][:] = [2, 2, 30]
+    w["L0"][:] = 20.0
+    w["gait_amp"][:] = 0.0
+    s = W.solver_settings(n_sub=2, iters=6, gravity=(0.0, 0.0, 0.0), contact=False, solver=solver, pcr_iters=6)
+    g, o = Sim(w, s), oracle.OracleSim(w, s)
+    tiny = np.float32(sign * 5e-38)
+    for k, N in enumerate(W.n_nodes(w)):
+        x = np.zeros((N, 3))
+        x[:-1, 0] = 20.0 * (np.arange(N - 1) - (N - 2))
+        x[-1] = (tiny, 20.0 * (1 if k else -1), 0.0)
+        x[:, 2] = 1.0
+        o.x[o.snake_nodes(k)] = x
+    g.set_state(pos=o.x.astype(np.float32))
+    g.step(1)
+    o.step(1)
+    st = g.state_host()
+    assert np.isfinite(st["pos"]).all()
+    assert (np.linalg.norm(st["pos"] - o.x, axis=1) / node_scale(w, o.x)).max() <= 1e-5
+    assert np.abs(o.x[o.snake_nodes(0)][0] - [-20.0, 0.0, 1.0]).max() > 1.0  # the bend opens
