@@ -60,36 +60,44 @@ __device__ __forceinline__ float atan_unit(float t) {
   p = fmaf(p, s, 9.999998808e-01f);
   return t * p;
 }
-// 1 / a for 1 < a < inf: the hardware's approximate reciprocal and one Newton step (rounded like
+// 1 / a for 1 < a: the hardware's approximate reciprocal and one Newton step (rounded like
 // the exact value unless that lies within ~2^-45 of a rounding boundary), without the
 // branches of the general correctly rounded reciprocal, which every pass would issue for
-// the rare steep angles.
+// the rare steep angles.  Of an infinite a the step gives 0 x inf = NaN instead of 0, for which
+// there are two remedies, with the same bits: SAT saturates the result to [0, 1], which turns
+// NaN into 0 and is part of the instruction, and otherwise atan2_bend caps its tangent.  (An
+// infinite tangent of an elevation needs none: a vertical segment has no gradient either.)
+// Neither costs what it issues, they move the compiler's schedule: us per env-step without /
+// with SAT / with the cap, one snake 138 / 139 / 141, 221 snakes to 1e-4 8530 / 8642 / 8862, but
+// 256 cantilevers to 1e-6 (one node per lane) 6333 / 6449 / 6304, 604 wheeled snakes
+// (anisotropic) 6928 / 6931 / 6819: hence kSat.
+template <int NPL, bool ANISO>
+constexpr bool kSat = !ANISO && NPL >= 2;
 __device__ __forceinline__ float rcp_approx(float a) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a));
   return y;
 }
+template <bool SAT>
 __device__ __forceinline__ float rcp_newton(float a) {
   const float y = rcp_approx(a);
-  return fmaf(fmaf(-a, y, 1.f), y, y);
+  const float r = fmaf(fmaf(-a, y, 1.f), y, y);
+  return SAT ? __saturatef(r) : r;
 }
-template <bool INF = false>  // INF: t may be infinite
+template <bool SAT, bool CAP>
 __device__ __forceinline__ float atan_any(float t) {
-  const float a = INF ? fminf(fabsf(t), 3.0e38f) : fabsf(t);
+  const float a = CAP ? fminf(fabsf(t), 3.0e38f) : fabsf(t);
   const bool big = a > 1.f;
-  const float p = atan_unit(big ? rcp_newton(a) : a);
+  const float p = atan_unit(big ? rcp_newton<SAT>(a) : a);
   return copysignf(big ? 1.57079632679489662f - p : p, t);
 }
 // atan2(y, x) for the bend angles from the same polynomial, without branches: atan(y / x),
-// shifted by +-pi for x < 0, +-pi/2 (0 for y = 0) on the axis x = 0.  (The library atan2f
-// would add a large body of code to every solver kernel for the rare angles beyond 90
-// degrees.)  The quotient overflows next to the axis, hence the cap: one instruction per bend
-// row and pass (us per env-step without / with it: one snake 139.8 / 143.3, 4096 snakes
-// 586 / 589, 256 cantilevers to 1e-6 6345 / 6315, 1500 wheeled snakes to 1e-4 15640 / 15240).
-// The elevation's tangent in make_seg is infinite only where a segment stands vertically and
-// has no gradient either.
+// shifted by +-pi for x < 0, +-pi/2 (0 for y = 0) on the axis x = 0, next to which the quotient
+// overflows.  (The library atan2f would add a large body of code to every solver kernel for
+// the rare angles beyond 90 degrees.)
+template <bool SAT = false>
 __device__ __forceinline__ float atan2_bend(float y, float x) {
-  float r = atan_any<true>(__fdividef(y, x));
+  float r = atan_any<SAT, !SAT>(__fdividef(y, x));
   r = (x < 0.f) ? r + copysignf(3.14159265358979323846f, y) : r;
   const float axis = (y == 0.f) ? 0.f : copysignf(1.57079632679489662f, y);
   return (x == 0.f) ? axis : r;
@@ -104,6 +112,7 @@ struct Seg {  // derived quantities of the segment from node i to node i+1
   float beta;         // elevation atan2(e_z, |e_h|) = asin(e_z / |e|)
 };
 
+template <bool SAT = false>
 __device__ __forceinline__ Seg make_seg(float ex, float ey, float ez, float L0) {
   Seg s;
   s.ex = ex; s.ey = ey; s.ez = ez;
@@ -120,7 +129,7 @@ __device__ __forceinline__ Seg make_seg(float ex, float ey, float ez, float L0) 
   s.gpx = -s.ez * s.ex * f;
   s.gpy = -s.ez * s.ey * f;
   s.gpz = h2 * f;
-  s.beta = atan_any(s.ez * ih);  // atan2(e_z, |e_h|), |e_h| > 0
+  s.beta = atan_any<SAT, false>(s.ez * ih);  // atan2(e_z, |e_h|), |e_h| > 0
   return s;
 }
 
@@ -458,7 +467,8 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     auto seg = [&](int u) {
       const float* ad = (u == 0) ? dxl : dx[u > 0 ? u - 1 : 0];
       const float* bd = (u == NPL) ? dxr : dx[u < NPL ? u : 0];
-      return make_seg(xd[u][0] + (bd[0] - ad[0]), xd[u][1] + (bd[1] - ad[1]), xd[u][2] + (bd[2] - ad[2]), L0);
+      return make_seg<kSat<NPL, ANISO>>(xd[u][0] + (bd[0] - ad[0]), xd[u][1] + (bd[1] - ad[1]),
+                                        xd[u][2] + (bd[2] - ad[2]), L0);
     };
     float acc[NPL][3], dl[NPL][6];
     float accL[3] = {0.f, 0.f, 0.f}, accR[3] = {0.f, 0.f, 0.f};
@@ -493,7 +503,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
       {
         const float cz = sp.ex * sc.ey - sp.ey * sc.ex;
         const float dh = sp.ex * sc.ex + sp.ey * sc.ey;
-        const float c = L0 * (atan2_bend(cz, dh) - th[j]);
+        const float c = L0 * (atan2_bend<kSat<NPL, ANISO>>(cz, dh) - th[j]);
         const float g0x = sp.gyx, g0y = sp.gyy;                     // node i-1
         const float g1x = -sp.gyx - sc.gyx, g1y = -sp.gyy - sc.gyy; // node i
         const float g2x = sc.gyx, g2y = sc.gyy;                     // node i+1
