@@ -312,7 +312,9 @@ SimStatus sim_fp32_fma_probe(float* out_dev, int n_blocks, int iters, void* stre
 #define MLP_NUM_PARAMS 19841
 typedef struct MlpHandle MlpHandle;
 
-/* Creates a network with all parameters zero, bound to `stream` (cudaStream_t). */
+/* Creates a network with all parameters zero, bound to `stream` (cudaStream_t).  A network
+ * holds 12 MB of device memory (mostly the training blocks' partial gradients, taken here
+ * so that no later call allocates). */
 SimStatus mlp_create(void* stream, MlpHandle** out);
 /* Sets / reads the FP32 parameter vector; setting also resets the Adam moments. */
 SimStatus mlp_set_params(MlpHandle* m, const float* params, int is_device);

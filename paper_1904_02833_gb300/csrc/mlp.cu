@@ -152,8 +152,9 @@ __device__ __forceinline__ bool group_or(int group, bool v) {
 // What bounds it: the tanh unit (192 evaluations per row keep it busy 60 % of the kernel) and
 // the queue in front of it; the epilogues' issue slots are 1215 thread instructions per row
 // (1827 before); DRAM moves 68 bytes per row, a quarter of the time.  Measured, a call on
-// 1,261,356 rows: 146 us with one tile per eight-warp block and two threads per row, 133 us
-// now; outputs bit for bit the same.
+// 1,261,356 rows: 146 us with one tile per eight-warp block and two threads per row, 135 us
+// now; outputs bit for bit the same.  Kernel alone (us before / now): 128 rows 8.9 / 9.0, 16384
+// 8.9 / 9.0, 38912 (a tile per block) 11.1 / 11.2, 77952 16.4 / 14.9, 400000 43.5 / 41.2.
 __global__ void __launch_bounds__(kInferThreads, 2) mlp_infer_kernel(const __nv_bfloat16* __restrict__ feat,
                                                                     long long rows, MlpDev w,
                                                                     float* __restrict__ out, int* err,
