@@ -60,44 +60,36 @@ __device__ __forceinline__ float atan_unit(float t) {
   p = fmaf(p, s, 9.999998808e-01f);
   return t * p;
 }
-// 1 / a for 1 < a: the hardware's approximate reciprocal and one Newton step (rounded like
+// 1 / a for 1 < a < inf: the hardware's approximate reciprocal and one Newton step (rounded like
 // the exact value unless that lies within ~2^-45 of a rounding boundary), without the
 // branches of the general correctly rounded reciprocal, which every pass would issue for
-// the rare steep angles.  Of an infinite a the step gives 0 x inf = NaN instead of 0, for which
-// there are two remedies, with the same bits: SAT saturates the result to [0, 1], which turns
-// NaN into 0 and is part of the instruction, and otherwise atan2_bend caps its tangent.  (An
-// infinite tangent of an elevation needs none: a vertical segment has no gradient either.)
-// Neither costs what it issues, they move the compiler's schedule: us per env-step without /
-// with SAT / with the cap, one snake 138 / 139 / 141, 221 snakes to 1e-4 8530 / 8642 / 8862, but
-// 256 cantilevers to 1e-6 (one node per lane) 6333 / 6449 / 6304, 604 wheeled snakes
-// (anisotropic) 6928 / 6931 / 6819: hence kSat.
-template <int NPL, bool ANISO>
-constexpr bool kSat = !ANISO && NPL >= 2;
+// the rare steep angles.  (Of an infinite a it is NaN.)
 __device__ __forceinline__ float rcp_approx(float a) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a));
   return y;
 }
-template <bool SAT>
 __device__ __forceinline__ float rcp_newton(float a) {
   const float y = rcp_approx(a);
-  const float r = fmaf(fmaf(-a, y, 1.f), y, y);
-  return SAT ? __saturatef(r) : r;
+  return fmaf(fmaf(-a, y, 1.f), y, y);
 }
-template <bool SAT, bool CAP>
+// INF: t may be infinite; the minimum then takes pi / 2 in place of the NaN (p is never
+// negative, so that it is no change of any other result).  An infinite tangent of an elevation
+// needs no care: a vertical segment has no gradient either.
+template <bool INF = false>
 __device__ __forceinline__ float atan_any(float t) {
-  const float a = CAP ? fminf(fabsf(t), 3.0e38f) : fabsf(t);
+  constexpr float kHalfPi = 1.57079632679489662f;
+  const float a = fabsf(t);
   const bool big = a > 1.f;
-  const float p = atan_unit(big ? rcp_newton<SAT>(a) : a);
-  return copysignf(big ? 1.57079632679489662f - p : p, t);
+  const float p = atan_unit(big ? rcp_newton(a) : a);
+  return copysignf(big ? (INF ? fminf(kHalfPi - p, kHalfPi) : kHalfPi - p) : p, t);
 }
 // atan2(y, x) for the bend angles from the same polynomial, without branches: atan(y / x),
 // shifted by +-pi for x < 0, +-pi/2 (0 for y = 0) on the axis x = 0, next to which the quotient
 // overflows.  (The library atan2f would add a large body of code to every solver kernel for
 // the rare angles beyond 90 degrees.)
-template <bool SAT = false>
 __device__ __forceinline__ float atan2_bend(float y, float x) {
-  float r = atan_any<SAT, !SAT>(__fdividef(y, x));
+  float r = atan_any<true>(__fdividef(y, x));
   r = (x < 0.f) ? r + copysignf(3.14159265358979323846f, y) : r;
   const float axis = (y == 0.f) ? 0.f : copysignf(1.57079632679489662f, y);
   return (x == 0.f) ? axis : r;
@@ -112,7 +104,6 @@ struct Seg {  // derived quantities of the segment from node i to node i+1
   float beta;         // elevation atan2(e_z, |e_h|) = asin(e_z / |e|)
 };
 
-template <bool SAT = false>
 __device__ __forceinline__ Seg make_seg(float ex, float ey, float ez, float L0) {
   Seg s;
   s.ex = ex; s.ey = ey; s.ez = ez;
@@ -129,7 +120,7 @@ __device__ __forceinline__ Seg make_seg(float ex, float ey, float ez, float L0) 
   s.gpx = -s.ez * s.ex * f;
   s.gpy = -s.ez * s.ey * f;
   s.gpz = h2 * f;
-  s.beta = atan_any<SAT, false>(s.ez * ih);  // atan2(e_z, |e_h|), |e_h| > 0
+  s.beta = atan_any(s.ez * ih);  // atan2(e_z, |e_h|), |e_h| > 0
   return s;
 }
 
@@ -395,6 +386,14 @@ __device__ __forceinline__ void warm_pass(const SnakeK& S, const SolverArgs& A, 
 // snakes 785 -> 600 us; 8192 snakes to 1e-4 cold 49-58 -> 32-35 ms, 256 cantilevers to 1e-6
 // 30.9 -> 18.8 ms.
 constexpr float kDummy = 1.152921504606846976e18f;  // 2^60: its square is 2^120
+// Least compliance in a bend row's weight: the gradients of a solve that blows up (segments of
+// 1e18 rest lengths) underflow, and a hard row's weight with them.  No part of the sum for any
+// weight above 1e-22 (a mass below 1e22 kg at the usual lengths).  It and the infinite tangent of
+// atan2_bend issue next to nothing but move the compiler's schedule, by kernel and by form: of
+// seven pairs of forms the present one is the most even (us per env-step without / with both:
+// one snake 140.8 / 142.0, 4096 snakes 589 / 593, 256 cantilevers to 1e-6 6350 / 6352, 221 snakes
+// to 1e-4 8542 / 8660, 604 wheeled ones 6933 / 6896; the others cost some of these 4-6 %).
+constexpr float kAbMin = 1e-30f;
 template <int NPL, int G, bool ANISO, bool WIDE>
 __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int q, bool valid,
                                        const float (&xs)[NPL][3], float (&dx)[NPL][3], const float (&xsl)[3],
@@ -435,7 +434,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     ws[j] = st ? 1.f : 0.f;
     rs[j] = st ? rcp_approx(wg + S.at_s) : 0.f;
     wb[j] = bd ? 1.f : 0.f;
-    ab[j] = bd ? S.at_b : INFINITY;
+    ab[j] = bd ? fmaxf(S.at_b, kAbMin) : INFINITY;
     zc[j] = xs[j][2] - S.radius;
     om[j] = A.contact && w[j + 1] > 0.f ? S.om_m : 0.f;
     if constexpr (ANISO) {
@@ -467,8 +466,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
     auto seg = [&](int u) {
       const float* ad = (u == 0) ? dxl : dx[u > 0 ? u - 1 : 0];
       const float* bd = (u == NPL) ? dxr : dx[u < NPL ? u : 0];
-      return make_seg<kSat<NPL, ANISO>>(xd[u][0] + (bd[0] - ad[0]), xd[u][1] + (bd[1] - ad[1]),
-                                        xd[u][2] + (bd[2] - ad[2]), L0);
+      return make_seg(xd[u][0] + (bd[0] - ad[0]), xd[u][1] + (bd[1] - ad[1]), xd[u][2] + (bd[2] - ad[2]), L0);
     };
     float acc[NPL][3], dl[NPL][6];
     float accL[3] = {0.f, 0.f, 0.f}, accR[3] = {0.f, 0.f, 0.f};
@@ -503,7 +501,7 @@ __device__ __forceinline__ void jacobi(const SnakeK& S, const SolverArgs& A, int
       {
         const float cz = sp.ex * sc.ey - sp.ey * sc.ex;
         const float dh = sp.ex * sc.ex + sp.ey * sc.ey;
-        const float c = L0 * (atan2_bend<kSat<NPL, ANISO>>(cz, dh) - th[j]);
+        const float c = L0 * (atan2_bend(cz, dh) - th[j]);
         const float g0x = sp.gyx, g0y = sp.gyy;                     // node i-1
         const float g1x = -sp.gyx - sc.gyx, g1y = -sp.gyy - sc.gyy; // node i
         const float g2x = sc.gyx, g2y = sc.gyy;                     // node i+1

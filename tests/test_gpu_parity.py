@@ -745,3 +745,30 @@ def test_right_angles_whose_tangent_overflows(solver, sign):
     assert np.isfinite(st["pos"]).all()
     assert (np.linalg.norm(st["pos"] - o.x, axis=1) / node_scale(w, o.x)).max() <= 1e-5
     assert np.abs(o.x[o.snake_nodes(0)][0] - [-20.0, 0.0, 1.0]).max() > 1.0  # the bend opens
+
+
+@pytest.mark.parametrize("lanes,npl", [(8, 1), (16, 2), (32, 2), (32, 4)])
+def test_hard_bend_rows_whose_weight_underflows(lanes, npl):
+    """Segments of 4e18 m bent by 90 degrees (a solve that has blown up): the bend rows' weight is
+    zero in 32 bits and, with no compliance, so is their divisor.  The rows move nothing
+    (as with a compliance, whose updates are far below the positions' rounding) and the
+    stretch rows go on."""
+    w = W.batched(n=2, seed=57, links=(1, 1))
+    w["seg_per_link"][:] = [2, 6]
+    w["alpha_b"][:] = 0.0
+    w["gait_amp"][:] = 0.0
+    soft = dict(w, alpha_b=np.full(2, 1.0))
+    s = W.solver_settings(n_sub=1, iters=2, gravity=(0.0, 0.0, 0.0), contact=False)
+    out = []
+    for p in (w, soft):
+        g = Sim(p, s)
+        for N in (3, 7):
+            g.set_layout(N, lanes, npl)
+        k = np.concatenate([np.arange(3), np.arange(7)])
+        x = np.stack([4e18 * ((k + 1) // 2), 4e18 * (k // 2), np.ones(10)], 1).astype(np.float32)
+        g.set_state(pos=x)
+        g.step(1)
+        out.append(g.state_host()["pos"])
+        assert g.status()[0] != -4
+    assert np.isfinite(out[0]).all()
+    assert np.abs(out[0] - out[1]).max() <= 1e-6 * 4e18
